@@ -5,8 +5,11 @@
 // assumes, and the serving loop's iterative request type.
 //
 // Norms and the Rayleigh quotient are FP64 two-stage reductions with a fixed
-// block split, so the result is deterministic.  The normalisation reads the
-// norm from device memory: no host round trip inside the loop.
+// block split and fixed trees, so the result is deterministic.  The
+// normalisation reads the norm from device memory: no host round trip inside
+// the loop.  A step is three launches: the product w = A v, the partial sums of
+// w.w (and of v.w for the quotient), and one kernel that adds the partials,
+// scales w and gathers the next product's x' = v[cperm].
 #include <algorithm>
 
 #include "handle.cuh"
@@ -17,83 +20,126 @@ namespace {
 constexpr int kDotThreads = 256;
 constexpr int kDotBlocks = 512;
 
+// Sum of v over the block (a fixed tree), valid in every thread; ws: one
+// double per warp.  Starts and ends with a barrier, so ws can be reused.
+__device__ __forceinline__ double block_sum(double v, double* ws) {
+#pragma unroll
+  for (int d = 16; d > 0; d >>= 1) v += __shfl_xor_sync(0xffffffffu, v, d);
+  __syncthreads();
+  if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = v;
+  __syncthreads();
+  double t = 0.0;
+#pragma unroll
+  for (int w = 0; w < kDotThreads / 32; ++w) t += ws[w];
+  return t;
+}
+
+// Sum of np <= kDotBlocks partials, valid in every thread of a block.
+__device__ __forceinline__ double sum_parts(const double* __restrict__ part, int np, double* ws) {
+  const int t = threadIdx.x;
+  double a = t < np ? part[t] : 0.0;
+  static_assert(kDotBlocks <= 2 * kDotThreads, "two partials per thread");
+  if (t + kDotThreads < np) a += part[t + kDotThreads];
+  return block_sum(a, ws);
+}
+
+// part_aa[b] = sum of a[i]^2, part_ab[b] = sum of a[i] * b[Qb ? Qb[i] : i] over
+// block b's slice (either may be null).  Four elements of a thread are in
+// flight at a time: at the served sizes the kernel is one or two rounds of
+// load latency, not bandwidth.
 template <typename T>
 __global__ void __launch_bounds__(kDotThreads) dot_partial(const T* __restrict__ a, const T* __restrict__ b,
-                                                           int64_t n, double* __restrict__ part) {
+                                                           const int32_t* __restrict__ Qb, int64_t n,
+                                                           double* __restrict__ part_aa,
+                                                           double* __restrict__ part_ab) {
+  __shared__ double ws[kDotThreads / 32];
   const int64_t per = (n + gridDim.x - 1) / gridDim.x;
   const int64_t lo = blockIdx.x * per, hi = std::min<int64_t>(n, lo + per);
-  double acc = 0.0;
-  for (int64_t i = lo + threadIdx.x; i < hi; i += kDotThreads)
-    acc += static_cast<double>(a[i]) * static_cast<double>(b[i]);
-  __shared__ double ws[kDotThreads / 32];
+  double aa = 0.0, ab = 0.0;
+  for (int64_t i0 = lo + threadIdx.x; i0 < hi; i0 += 4 * kDotThreads) {
+    T x[4], y[4];
 #pragma unroll
-  for (int d = 16; d > 0; d >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, d);
-  if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = acc;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double t = 0.0;
-    for (int w = 0; w < kDotThreads / 32; ++w) t += ws[w];
-    part[blockIdx.x] = t;
-  }
-}
-
-__global__ void dot_final(const double* __restrict__ part, int nparts, double* __restrict__ out) {
-  if (threadIdx.x == 0 && blockIdx.x == 0) {
-    double t = 0.0;
-    for (int i = 0; i < nparts; ++i) t += part[i];
-    *out = t;
-  }
-}
-
-template <typename T>
-__global__ void scale_by_inv_norm(const T* __restrict__ w, const double* __restrict__ nrm2, int64_t n,
-                                  T* __restrict__ v) {
-  const int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const double inv = 1.0 / sqrt(*nrm2);
-  v[i] = static_cast<T>(static_cast<double>(w[i]) * inv);
-}
-
-// out[j] = w[Q[j]] * (1 / sqrt(*nrm2))
-template <typename T>
-__global__ void gather_scale(const int32_t* __restrict__ Q, const T* __restrict__ w, const double* __restrict__ nrm2,
-                             int64_t n, T* __restrict__ out) {
-  const int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const double inv = 1.0 / sqrt(*nrm2);
-  const int64_t src = Q ? static_cast<int64_t>(Q[i]) : i;
-  out[i] = static_cast<T>(static_cast<double>(w[src]) * inv);
-}
-
-// part[b] = sum over block b's slice of u[i] * w[Q[i]]
-template <typename T>
-__global__ void __launch_bounds__(kDotThreads) dot_gather_partial(const T* __restrict__ u, const T* __restrict__ w,
-                                                                  const int32_t* __restrict__ Q, int64_t n,
-                                                                  double* __restrict__ part) {
-  const int64_t per = (n + gridDim.x - 1) / gridDim.x;
-  const int64_t lo = blockIdx.x * per, hi = std::min<int64_t>(n, lo + per);
-  double acc = 0.0;
-  for (int64_t i = lo + threadIdx.x; i < hi; i += kDotThreads)
-    acc += static_cast<double>(u[i]) * static_cast<double>(w[Q ? static_cast<int64_t>(Q[i]) : i]);
-  __shared__ double ws[kDotThreads / 32];
+    for (int u = 0; u < 4; ++u) {
+      const int64_t i = i0 + u * kDotThreads;
+      x[u] = i < hi ? a[i] : T(0);
+      y[u] = part_ab && i < hi ? b[Qb ? static_cast<int64_t>(Qb[i]) : i] : T(0);
+    }
 #pragma unroll
-  for (int d = 16; d > 0; d >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, d);
-  if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = acc;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double t = 0.0;
-    for (int k = 0; k < kDotThreads / 32; ++k) t += ws[k];
-    part[blockIdx.x] = t;
+    for (int u = 0; u < 4; ++u) {
+      if (part_aa) aa = fma(static_cast<double>(x[u]), static_cast<double>(x[u]), aa);
+      if (part_ab) ab = fma(static_cast<double>(x[u]), static_cast<double>(y[u]), ab);
+    }
+  }
+  if (part_aa) {
+    const double t = block_sum(aa, ws);
+    if (threadIdx.x == 0) part_aa[blockIdx.x] = t;
+  }
+  if (part_ab) {
+    const double t = block_sum(ab, ws);
+    if (threadIdx.x == 0) part_ab[blockIdx.x] = t;
   }
 }
 
+// One block: *out = the sum of the partials.  One thread adding them in turn
+// took 21 us (512 dependent FP64 adds behind loads).
+__global__ void __launch_bounds__(kDotThreads) dot_final(const double* __restrict__ part, int nparts,
+                                                         double* __restrict__ out) {
+  __shared__ double ws[kDotThreads / 32];
+  const double t = sum_parts(part, nparts, ws);
+  if (threadIdx.x == 0) *out = t;
+}
+
+constexpr int kScaleItems = 4;  // elements per thread
+
+// With s = the sum of part_ww (every block adds the same partials in the same
+// order, so no block waits for another): out[j] = w[Q ? Q[j] : j] / sqrt(s)
+// and v[j] = w[j] / sqrt(s) (out or v may be null).  Block 0 also writes s to
+// *nrm2 and the sum of part_vw to *vw (either may be null).  The square root
+// and the division are done once per block: in FP64, with two FMA lanes per SM,
+// one of each per element took 12 us of a 300 k vector's step.
 template <typename T>
-maxe_status dot(const T* a, const T* b, int64_t n, double* part, double* out, cudaStream_t st) {
-  const int nb = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(kDotBlocks, ceil_div(n, 4 * kDotThreads))));
-  dot_partial<T><<<nb, kDotThreads, 0, st>>>(a, b, n, part);
-  dot_final<<<1, 32, 0, st>>>(part, nb, out);
-  MAXE_CUDA_TRY(cudaGetLastError());
-  return MAXE_OK;
+__global__ void __launch_bounds__(kDotThreads) scale_gather(const int32_t* __restrict__ Q, const T* __restrict__ w,
+                                                            const double* __restrict__ part_ww,
+                                                            const double* __restrict__ part_vw, int np, int64_t n,
+                                                            T* __restrict__ out, T* __restrict__ v,
+                                                            double* __restrict__ nrm2, double* __restrict__ vw) {
+  __shared__ double ws[kDotThreads / 32];
+  __shared__ double inv_s;
+  const int64_t i0 = static_cast<int64_t>(blockIdx.x) * (kDotThreads * kScaleItems) + threadIdx.x;
+  T g[kScaleItems], own[kScaleItems];
+#pragma unroll
+  for (int u = 0; u < kScaleItems; ++u) {  // the loads fly while the partials are added
+    const int64_t i = i0 + u * kDotThreads;
+    g[u] = out && i < n ? w[Q ? static_cast<int64_t>(Q[i]) : i] : T(0);
+    own[u] = v && i < n ? w[i] : T(0);
+  }
+  const double s = sum_parts(part_ww, np, ws);
+  if (threadIdx.x == 0) {
+    inv_s = 1.0 / sqrt(s);
+    if (blockIdx.x == 0 && nrm2) *nrm2 = s;
+  }
+  if (blockIdx.x == 0 && vw) {
+    const double q = sum_parts(part_vw, np, ws);
+    if (threadIdx.x == 0) *vw = q;
+  }
+  __syncthreads();
+  const double inv = inv_s;
+#pragma unroll
+  for (int u = 0; u < kScaleItems; ++u) {
+    const int64_t i = i0 + u * kDotThreads;
+    if (i < n) {
+      if (out) out[i] = static_cast<T>(static_cast<double>(g[u]) * inv);
+      if (v) v[i] = static_cast<T>(static_cast<double>(own[u]) * inv);
+    }
+  }
+}
+
+int dot_blocks(int64_t n) {
+  return static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(kDotBlocks, ceil_div(n, 4 * kDotThreads))));
+}
+
+unsigned scale_blocks(int64_t n) {
+  return static_cast<unsigned>(std::max<int64_t>(1, ceil_div(n, kDotThreads * kScaleItems)));
 }
 
 // hist_host (nullable): the Rayleigh quotient v^T A v of the iterate after
@@ -105,31 +151,30 @@ maxe_status run(const maxe_handle* h, const T* v0, int32_t steps, T* v, double* 
   const int64_t n = h->rows;
   ScratchSet scratch(h->al);
   T* w = scratch.get<T>(static_cast<size_t>(n));
-  T* xp = scratch.get<T>(static_cast<size_t>(n));
-  double* part = scratch.get<double>(kDotBlocks + 2 + (hist_host ? std::max(steps, 1) : 0));
-  if (!w || !xp || !part) return MAXE_ERR_OOM;
-  double* nrm2 = part + kDotBlocks;
-  double* lam = part + kDotBlocks + 1;
-  double* hist = hist_host ? part + kDotBlocks + 2 : nullptr;
+  T* xp = h->cperm ? scratch.get<T>(static_cast<size_t>(n)) : nullptr;
+  double* part = scratch.get<double>(2 * kDotBlocks + 1 + (hist_host ? std::max(steps, 1) : 0));
+  if (!w || (h->cperm && !xp) || !part) return MAXE_ERR_OOM;
+  double* part_vw = part + kDotBlocks;
+  double* lam = part_vw + kDotBlocks;
+  double* hist = hist_host ? lam + 1 : nullptr;
   MAXE_CUDA_TRY(cudaMemcpyAsync(v, v0, sizeof(T) * n, cudaMemcpyDeviceToDevice, st));
-  const unsigned grid = static_cast<unsigned>(std::max<int64_t>(1, ceil_div(n, 256)));
-  auto product = [&](const T* x, T* y) -> maxe_status {
-    const T* xs = x;
-    if (h->cperm) {
-      MAXE_TRY(launch_gather(h->cperm, n, sizeof(T), 1, x, 1, xp, 1, st));
-      xs = xp;
-    }
-    return spmm_launch(h, 1, xs, 1, y, 1, h->rperm, st);
-  };
+  if (xp) MAXE_TRY(launch_gather(h->cperm, n, sizeof(T), 1, v0, 1, xp, 1, st));
+  const int nb = dot_blocks(n);
+  const T* x = xp ? xp : v;  // the product's x': v itself on a matrix whose columns were not permuted
   for (int32_t s = 0; s < steps; ++s) {
-    MAXE_TRY(product(v, w));
-    if (hist && s > 0) MAXE_TRY(dot(v, w, n, part, hist + s - 1, st));  // v = the iterate after step s
-    MAXE_TRY(dot(w, w, n, part, nrm2, st));
-    scale_by_inv_norm<T><<<grid, 256, 0, st>>>(w, nrm2, n, v);
+    MAXE_TRY(spmm_launch(h, 1, x, 1, w, 1, h->rperm, st));
+    const bool quotient = hist && s > 0;  // v = the iterate after step s
+    dot_partial<T><<<nb, kDotThreads, 0, st>>>(w, v, nullptr, n, part, quotient ? part_vw : nullptr);
+    const bool need_v = !xp || hist || s + 1 == steps;  // v besides the gathered x'
+    scale_gather<T><<<scale_blocks(n), kDotThreads, 0, st>>>(h->cperm, w, part, part_vw, nb, n, xp,
+                                                             need_v ? v : nullptr, nullptr,
+                                                             quotient ? hist + s - 1 : nullptr);
     MAXE_CUDA_TRY(cudaGetLastError());
   }
-  MAXE_TRY(product(v, w));
-  MAXE_TRY(dot(v, w, n, part, lam, st));
+  MAXE_TRY(spmm_launch(h, 1, x, 1, w, 1, h->rperm, st));
+  dot_partial<T><<<nb, kDotThreads, 0, st>>>(v, w, nullptr, n, nullptr, part_vw);
+  dot_final<<<1, kDotThreads, 0, st>>>(part_vw, nb, lam);
+  MAXE_CUDA_TRY(cudaGetLastError());
   MAXE_CUDA_TRY(cudaMemcpyAsync(lambda_host, lam, sizeof(double), cudaMemcpyDeviceToHost, st));
   if (hist && steps > 0) {
     if (steps > 1)
@@ -140,17 +185,12 @@ maxe_status run(const maxe_handle* h, const T* v0, int32_t steps, T* v, double* 
   return MAXE_OK;
 }
 
-int dot_blocks(int64_t n) {
-  return static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(kDotBlocks, ceil_div(n, 4 * kDotThreads))));
-}
-
 template <typename T>
 maxe_status norm_gather(const int32_t* Q, int64_t n, const T* w, T* u, double* scratch, cudaStream_t st) {
   const int nb = dot_blocks(n);
-  dot_partial<T><<<nb, kDotThreads, 0, st>>>(w, w, n, scratch);
-  dot_final<<<1, 32, 0, st>>>(scratch, nb, scratch + kDotBlocks);
-  gather_scale<T><<<static_cast<unsigned>(std::max<int64_t>(1, ceil_div(n, 256))), 256, 0, st>>>(
-      Q, w, scratch + kDotBlocks, n, u);
+  dot_partial<T><<<nb, kDotThreads, 0, st>>>(w, nullptr, nullptr, n, scratch, nullptr);
+  scale_gather<T><<<scale_blocks(n), kDotThreads, 0, st>>>(Q, w, scratch, nullptr, nb, n, u, nullptr,
+                                                           scratch + kDotBlocks, nullptr);
   MAXE_CUDA_TRY(cudaGetLastError());
   return MAXE_OK;
 }
@@ -159,8 +199,8 @@ template <typename T>
 maxe_status dot_gather(const int32_t* Q, int64_t n, const T* u, const T* w, double* scratch, double* out,
                        cudaStream_t st) {
   const int nb = dot_blocks(n);
-  dot_gather_partial<T><<<nb, kDotThreads, 0, st>>>(u, w, Q, n, scratch);
-  dot_final<<<1, 32, 0, st>>>(scratch, nb, out);
+  dot_partial<T><<<nb, kDotThreads, 0, st>>>(u, w, Q, n, nullptr, scratch);
+  dot_final<<<1, kDotThreads, 0, st>>>(scratch, nb, out);
   MAXE_CUDA_TRY(cudaGetLastError());
   return MAXE_OK;
 }
