@@ -260,7 +260,7 @@ MAXE_API maxe_status maxe_entropy_levels(const int64_t* counts_dev, int32_t gr, 
  * input and output buffers, or code on a path where cudaMalloc's implicit
  * device-wide synchronisation is not allowed.  This entry point computes the
  * same counts and H as maxe_nnz_entropy, and allocates nothing: its scratch is
- * a static device array of 65536 32-bit counts plus one double (256 KiB),
+ * a static device array of 65537 32-bit counts plus 513 doubles (260 KiB),
  * which every GPU that loads the library holds until the process exits.
  * Arguments as for maxe_nnz_entropy (there is no allocator argument).
  * Limits and behaviour:
