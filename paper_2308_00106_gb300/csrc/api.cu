@@ -131,13 +131,9 @@ maxe_status maxe_build_permutation(uint64_t seed, int32_t n, int32_t tag, int32_
   cudaStream_t st = as_stream(stream);
   Allocator al(alloc, st);
   ScratchSet scratch(al);
-  uint64_t* keys = scratch.get<uint64_t>(n);
-  uint64_t* keys_alt = scratch.get<uint64_t>(n);
-  int32_t* vals_alt = scratch.get<int32_t>(n);
-  void* rs = scratch.get<unsigned char>(radix_scratch_bytes(n));
-  if (!keys || !keys_alt || !vals_alt || !rs) return MAXE_ERR_OOM;
-  MAXE_TRY(launch_keys(seed, n, tag, keys, perm, st));
-  return radix_sort_pairs(keys, perm, keys_alt, vals_alt, n, 64, rs, st);
+  void* tmp = scratch.get<unsigned char>(perm_order_scratch_bytes(n));
+  if (!tmp) return MAXE_ERR_OOM;
+  return perm_order(seed, tag, 0, n, perm, tmp, st);
 }
 
 maxe_status maxe_nnz_histogram(const maxe_csr* A, int32_t axis, int32_t* hist, void* stream) {

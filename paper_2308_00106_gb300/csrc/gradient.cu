@@ -9,14 +9,14 @@
 //              reduced with atomicMax, so the first steepest step wins whatever
 //              the schedule; the cut is before element i+1.
 //   order:     each half of the deck is sorted by the Section 3 keys of its
-//              positions (the radix sort of perm.cu, once per half).
+//              positions (perm_order of perm.cu, once per half).
 //   compose:   perm[new] = deck[order[new]], the riffle written in closed form:
 //              with parts of a = pivot and b = n - pivot cards and m = min(a, b),
 //              deck[d] = d/2 (d even) or pivot + d/2 (d odd) for d < 2m, then the
 //              longer part's remainder in order.
 #include <algorithm>
 
-#include "internal.cuh"
+#include "handle.cuh"
 
 namespace maxe {
 namespace {
@@ -93,22 +93,19 @@ maxe_status gradient_permutation_run(const int32_t* hist, int32_t n, uint64_t se
   if (n == 0) return pivot_out ? set_i32(pivot_out, 0, st) : MAXE_OK;
   const int32_t half = (n + 1) / 2;
   ScratchSet scratch(al);
-  uint64_t* keys = scratch.get<uint64_t>(n);
-  uint64_t* keys_alt = scratch.get<uint64_t>(half);
   int32_t* order = scratch.get<int32_t>(n);
-  int32_t* vals_alt = scratch.get<int32_t>(half);
-  void* rs = scratch.get<unsigned char>(radix_scratch_bytes(half));
+  void* tmp = scratch.get<unsigned char>(perm_order_scratch_bytes(half));
   unsigned long long* best = scratch.get<unsigned long long>(1);
-  if (!keys || !keys_alt || !order || !vals_alt || !rs || !best) return MAXE_ERR_OOM;
+  if (!order || !tmp || !best) return MAXE_ERR_OOM;
   MAXE_CUDA_TRY(cudaMemsetAsync(best, 0, sizeof(unsigned long long), st));
   if (n >= 2) {
     const int64_t blocks = std::min<int64_t>(ceil_div(n, kThreads), 152 * 8);
     steepest_kernel<<<static_cast<unsigned>(blocks), kThreads, 0, st>>>(hist, n, best);
     MAXE_CUDA_TRY(cudaGetLastError());
   }
-  MAXE_TRY(launch_keys(seed, n, tag, keys, order, st));  // keys of the deck positions, order = positions
-  MAXE_TRY(radix_sort_pairs(keys, order, keys_alt, vals_alt, half, 64, rs, st));
-  MAXE_TRY(radix_sort_pairs(keys + half, order + half, keys_alt, vals_alt, n - half, 64, rs, st));
+  // the deck positions of each half by their keys
+  MAXE_TRY(perm_order(seed, tag, 0, half, order, tmp, st));
+  MAXE_TRY(perm_order(seed, tag, half, n - half, order + half, tmp, st));
   riffle_compose_kernel<<<static_cast<unsigned>(ceil_div(n, kThreads)), kThreads, 0, st>>>(order, n, best, perm,
                                                                                          pivot_out);
   MAXE_CUDA_TRY(cudaGetLastError());

@@ -74,6 +74,11 @@ namespace maxe {
 inline int value_bytes(maxe_dtype d) { return d == MAXE_F64 ? 8 : (d == MAXE_F32 ? 4 : 2); }
 inline int vector_bytes(maxe_dtype d) { return d == MAXE_F64 ? 8 : 4; }
 
+// perm.cu: out = first .. first + n - 1 in ascending (key(seed, tag, i), i) order.
+size_t perm_order_scratch_bytes(int64_t n);
+maxe_status perm_order(uint64_t seed, int32_t tag, int32_t first, int32_t n, int32_t* out, void* scratch,
+                       cudaStream_t st);
+
 // spmv.cu
 int64_t spmv_pad_elems();
 maxe_status spmv_build_partition(maxe_handle* h, cudaStream_t st);
