@@ -344,13 +344,69 @@ __global__ void invert_kernel(const int32_t* __restrict__ perm, int32_t n, int32
   if (i < n) inv[perm[i]] = static_cast<int32_t>(i);
 }
 
+constexpr int kGatherThreads = 256;
+constexpr int kGatherRows = 4;  // rows per thread, their loads in flight together
+
+// out row i = in row perm[i], row_elems elements each, in pieces of V = VE
+// elements (16 bytes where the rows are aligned, else one element): a group of
+// 2^shift lanes takes a row, piece after piece, and a thread has kGatherRows
+// rows in flight.  Bound by the random reads of `in`: a 16-byte row still
+// moves a 32-byte sector (4.19M rows of 4 FP32: 16 us of sectors and 20 us of
+// the rest at 6.8 TB/s).  One element per thread with a 64-bit division to
+// find its row took 87 us there.
+template <typename T, typename V>
+__global__ void __launch_bounds__(kGatherThreads) gather_kernel(const int32_t* __restrict__ perm, int64_t n,
+                                                                int row_elems, int shift, const T* __restrict__ in,
+                                                                int64_t ld_in, T* __restrict__ out, int64_t ld_out) {
+  constexpr int VE = sizeof(V) / sizeof(T);
+  const int rows = kGatherThreads >> shift;  // per step of the block
+  const int c0 = (threadIdx.x & ((1 << shift) - 1)) * VE;
+  const int64_t i0 = static_cast<int64_t>(blockIdx.x) * rows * kGatherRows + (threadIdx.x >> shift);
+  int64_t src[kGatherRows];
+#pragma unroll
+  for (int u = 0; u < kGatherRows; ++u) {
+    const int64_t i = i0 + u * rows;
+    src[u] = i < n ? static_cast<int64_t>(perm[i]) * ld_in : 0;
+  }
+  for (int c = c0; c < row_elems; c += VE << shift) {
+    if (c + VE <= row_elems) {
+      V v[kGatherRows];
+#pragma unroll
+      for (int u = 0; u < kGatherRows; ++u)
+        if (i0 + u * rows < n) v[u] = *reinterpret_cast<const V*>(in + src[u] + c);
+#pragma unroll
+      for (int u = 0; u < kGatherRows; ++u)
+        if (i0 + u * rows < n) *reinterpret_cast<V*>(out + (i0 + u * rows) * ld_out + c) = v[u];
+    } else {  // the row's last piece, shorter: its elements alone
+      for (int u = 0; u < kGatherRows; ++u)
+        if (i0 + u * rows < n)
+          for (int e = c; e < row_elems; ++e) out[(i0 + u * rows) * ld_out + e] = in[src[u] + e];
+    }
+  }
+}
+
+template <typename T, typename V>
+void gather_launch(const int32_t* perm, int64_t n, int64_t row_elems, const void* in, int64_t ld_in, void* out,
+                   int64_t ld_out, cudaStream_t st) {
+  constexpr int VE = sizeof(V) / sizeof(T);
+  int shift = 0;  // lanes per row: a power of two, at most 32
+  while (shift < 5 && (static_cast<int64_t>(VE) << shift) < row_elems) ++shift;
+  const int64_t rows = static_cast<int64_t>(kGatherThreads >> shift) * kGatherRows;
+  gather_kernel<T, V><<<static_cast<unsigned>(ceil_div(n, rows)), kGatherThreads, 0, st>>>(
+      perm, n, static_cast<int>(row_elems), shift, static_cast<const T*>(in), ld_in, static_cast<T*>(out), ld_out);
+}
+
+// 16-byte pieces when rows of more than one element start on 16-byte boundaries on both sides.
 template <typename T>
-__global__ void gather_kernel(const int32_t* __restrict__ perm, int64_t n, int64_t row_elems,
-                              const T* __restrict__ in, int64_t ld_in, T* __restrict__ out, int64_t ld_out) {
-  const int64_t t = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (t >= n * row_elems) return;
-  const int64_t i = t / row_elems, c = t - i * row_elems;
-  out[i * ld_out + c] = in[static_cast<int64_t>(perm[i]) * ld_in + c];
+void gather_any(const int32_t* perm, int64_t n, int64_t row_elems, const void* in, int64_t ld_in, void* out,
+                int64_t ld_out, cudaStream_t st) {
+  constexpr int64_t VE = 16 / sizeof(T);
+  const bool wide = row_elems > 1 && ld_in % VE == 0 && ld_out % VE == 0 &&
+                    ((reinterpret_cast<uintptr_t>(in) | reinterpret_cast<uintptr_t>(out)) & 15u) == 0;
+  if (wide)
+    gather_launch<T, uint4>(perm, n, row_elems, in, ld_in, out, ld_out, st);
+  else
+    gather_launch<T, T>(perm, n, row_elems, in, ld_in, out, ld_out, st);
 }
 
 template <typename T>
@@ -448,24 +504,12 @@ maxe_status launch_invert(const int32_t* perm, int32_t n, int32_t* inv, cudaStre
 
 maxe_status launch_gather(const int32_t* perm, int64_t n, int elem_bytes, int64_t row_elems, const void* in,
                           int64_t ld_in, void* out, int64_t ld_out, cudaStream_t st) {
-  const int64_t total = n * row_elems;
-  if (total <= 0) return MAXE_OK;
-  const unsigned grid = static_cast<unsigned>(ceil_div(total, 256));
+  if (n <= 0 || row_elems <= 0) return MAXE_OK;
   switch (elem_bytes) {
-    case 2:
-      gather_kernel<uint16_t><<<grid, 256, 0, st>>>(perm, n, row_elems, static_cast<const uint16_t*>(in), ld_in,
-                                                   static_cast<uint16_t*>(out), ld_out);
-      break;
-    case 4:
-      gather_kernel<uint32_t><<<grid, 256, 0, st>>>(perm, n, row_elems, static_cast<const uint32_t*>(in), ld_in,
-                                                   static_cast<uint32_t*>(out), ld_out);
-      break;
-    case 8:
-      gather_kernel<uint64_t><<<grid, 256, 0, st>>>(perm, n, row_elems, static_cast<const uint64_t*>(in), ld_in,
-                                                   static_cast<uint64_t*>(out), ld_out);
-      break;
-    default:
-      return MAXE_ERR_INVALID;
+    case 2: gather_any<uint16_t>(perm, n, row_elems, in, ld_in, out, ld_out, st); break;
+    case 4: gather_any<uint32_t>(perm, n, row_elems, in, ld_in, out, ld_out, st); break;
+    case 8: gather_any<uint64_t>(perm, n, row_elems, in, ld_in, out, ld_out, st); break;
+    default: return MAXE_ERR_INVALID;
   }
   MAXE_CUDA_TRY(cudaGetLastError());
   return MAXE_OK;
