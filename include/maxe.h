@@ -231,7 +231,8 @@ MAXE_API maxe_status maxe_handle_csr(const maxe_handle* h, maxe_csr* view_out, c
  * plus 0x40000 when the one-row-per-lane-group SpMM prefetches each lane
  * group's next X rows into L2 (picked by MAXE_AUTOTUNE: it pays where
  * neighbouring rows share X rows, as in a stencil, and costs on permuted
- * matrices).  items: (host). */
+ * matrices), plus 0x80000 when maxe_spmv stages the gathered x of a tile of
+ * rows in shared memory instead (picked by MAXE_AUTOTUNE; see maxe_spmv_tiles).  items: (host). */
 MAXE_API maxe_status maxe_handle_tuning(const maxe_handle* h, int32_t* items);
 
 /* a4.  Entropy of the nonzero distribution (Section 4, entropy equation;
@@ -286,6 +287,13 @@ MAXE_API maxe_status maxe_nnz_entropy_noalloc(const maxe_handle* h, int32_t gr, 
  * handles, FP32 otherwise.  x and y must not overlap.  Calls on one handle
  * without MAXE_VEC_PERMUTED share its x' scratch: do not overlap them in time. */
 MAXE_API maxe_status maxe_spmv(const maxe_handle* h, const void* x, void* y, uint32_t flags, void* stream);
+
+/* a6 + a5 by the staged-tile kernel, whichever kernel maxe_spmv takes for this
+ * handle: a CTA gathers x for a tile of whole rows into shared memory and sums
+ * the rows from there.  Arguments and result as for maxe_spmv.  UNSUPPORTED on
+ * a handle without tiles: they are cut by MAXE_AUTOTUNE (without
+ * MAXE_EQUAL_ROWS, on matrices with nonzeros). */
+MAXE_API maxe_status maxe_spmv_tiles(const maxe_handle* h, const void* x, void* y, uint32_t flags, void* stream);
 
 /* a6 + a5 from host memory (Section 2, CSR product): enqueues on `stream`, in
  * this order, the copy of x_host into x_dev, maxe_spmv(h, x_dev, y_dev, flags,

@@ -79,6 +79,7 @@ void release(maxe_handle* h) {
   const Allocator& al = h->al;
   al.put(h->xbuf);
   xslice_release(h);
+  al.put(h->tile);
   al.put(h->coo_carry);
   al.put(h->coo_row);
   al.put(h->bwrow);
@@ -209,6 +210,10 @@ maxe_status maxe_permute_csr(const maxe_csr* A, const int32_t* rperm, const int3
       s = MAXE_OK;
     }
   }
+  if (s == MAXE_OK && (flags & MAXE_AUTOTUNE) && !h->equal_rows) {
+    s = spmv_tile_build(h, st);
+    if (s == MAXE_ERR_OOM) s = MAXE_OK;  // as above: the handle goes without it
+  }
   if (s == MAXE_OK) s = batch_plan_default(h, st);
   if (s == MAXE_OK && (flags & MAXE_ITEMS16)) h->spmv_items16 = 1;
   if (s == MAXE_OK && (flags & MAXE_SPMM_LANES)) h->spmm_lc = 1;
@@ -245,7 +250,7 @@ maxe_status maxe_handle_tuning(const maxe_handle* h, int32_t* items) {
   *items = (h->spmv_items16 ? 16 : 8) | (h->spmm_lc ? 0x100 : 0) | (h->xs_use ? 0x200 : 0) |
            (h->xs_use && h->xs_prefetch ? 0x400 : 0) | (h->xs_use && h->xs_pair == 2 ? 0x800 : 0) |
            (h->spmm_rows ? 0x1000 : 0) | ((h->blc & 3) << 13) | (((h->xs_ahead / 512) & 7) << 15) |
-           (h->spmm_rows_pf ? 0x40000 : 0);
+           (h->spmm_rows_pf ? 0x40000 : 0) | (h->tile_use ? 0x80000 : 0);
   return MAXE_OK;
 }
 
@@ -269,6 +274,20 @@ maxe_status maxe_spmv(const maxe_handle* h, const void* x, void* y, uint32_t fla
     xs = h->xbuf;
   }
   return spmm_launch(h, 1, xs, 1, y, 1, h->rperm, st);
+}
+
+maxe_status maxe_spmv_tiles(const maxe_handle* h, const void* x, void* y, uint32_t flags, void* stream) {
+  if (!h || flags & ~static_cast<uint32_t>(MAXE_VEC_PERMUTED)) return MAXE_ERR_INVALID;
+  if ((h->cols > 0 && !x) || (h->rows > 0 && !y)) return MAXE_ERR_INVALID;
+  if (!h->tiles) return MAXE_ERR_UNSUPPORTED;
+  cudaStream_t st = as_stream(stream);
+  if (flags & MAXE_VEC_PERMUTED) return spmv_tile_launch(h, x, y, nullptr, st);
+  const void* xs = x;
+  if (h->cperm) {
+    MAXE_TRY(launch_gather(h->cperm, h->cols, vector_bytes(h->dtype), 1, x, 1, h->xbuf, 1, st));
+    xs = h->xbuf;
+  }
+  return spmv_tile_launch(h, xs, y, h->rperm, st);
 }
 
 maxe_status maxe_spmv_host(const maxe_handle* h, const void* x_host, void* y_host, void* x_dev, void* y_dev,

@@ -32,6 +32,10 @@ struct maxe_handle {
   int spmm_rows = 0;                       // SpMM with one row per lane group (autotuned or 0)
   int spmm_rows_pf = 0;                    // that kernel prefetches each group's next X rows (autotuned)
   int equal_rows = 0;                      // SpMV partition: equal rows per warp (not equal nonzeros)
+  int2* tile = nullptr;                    // staged-tile SpMV (MAXE_AUTOTUNE): [tiles + 1] first row, its first entry
+  int64_t tiles = 0;
+  int tile_shift = 0;                      // log2 of its lanes per row
+  int tile_use = 0;                        // SpMV (k = 1) takes the staged-tile kernel (autotuned)
   int32_t* bwrow = nullptr;                // batch plan: partition with bH entries per warp task
   int32_t bnW = 0;
   int64_t bH = 0;
@@ -84,12 +88,18 @@ int64_t spmv_pad_elems();
 maxe_status spmv_build_partition(maxe_handle* h, cudaStream_t st);
 // Y = A' X (rows of Y optionally scattered through yperm).  X: cols x k (ldx),
 // Y: rows x k (ldy), vector element type of the handle.
-// variant: -1 = the handle's choice, 0 / 1 = force 8 / 16 entries per lane;
+// variant: -1 = the handle's choice, -2 = that without the staged tiles, 0 / 1 =
+// force 8 / 16 entries per lane;
 // lc: -1 = the handle's choice, 0 / 1 = force column passes / columns across lanes.
 maxe_status spmm_launch(const maxe_handle* h, int32_t k, const void* X, int64_t ldx, void* Y, int64_t ldy,
                         const int32_t* yperm, cudaStream_t st, int variant = -1, int lc = -1);
 // Time the SpMV variants on this matrix and keep the faster (synchronises).
 maxe_status spmv_autotune(maxe_handle* h, cudaStream_t st);
+
+// spmv_tile.cu: cut the rows into tiles; launch y' = A' x' over them (rows of y
+// optionally scattered through yperm).
+maxe_status spmv_tile_build(maxe_handle* h, cudaStream_t st);
+maxe_status spmv_tile_launch(const maxe_handle* h, const void* x, void* y, const int32_t* yperm, cudaStream_t st);
 
 // batch.cu
 constexpr int64_t kDefaultBatchTask = 2048;  // entries per warp task of the default batch plan

@@ -182,6 +182,7 @@ maxe_status spmm_launch(const maxe_handle* h, int32_t k, const void* X, int64_t 
       vw = 2;
   }
   const bool unit = k == 1 && ldx == 1 && ldy == 1;
+  if (unit && variant == -1 && lc < 0 && h->tile_use) return spmv_tile_launch(h, X, Y, yperm, st);
   if (unit && variant < 0 && lc < 0 && xslice_ready(h, X)) return xslice_launch(h, X, Y, yperm, st);
   if (k > 1 && variant < 0 && lc < 0 && h->spmm_rows && spmm_rows_ready(h, k, X, ldx, Y, ldy))
     return spmm_rows_launch(h, k, X, ldx, Y, ldy, yperm, st);
@@ -259,6 +260,14 @@ maxe_status spmv_autotune(maxe_handle* h, cudaStream_t st) {
     }
     h->xs_ahead = pick_d;
     if (s == MAXE_OK) h->xs_use = best_xs < best ? 1 : 0;
+    best = std::min(best, best_xs);
+  }
+  // the staged-tile kernel, when the handle has its tiles and it is clearly the
+  // faster (on small matrices all take a launch, and a tie keeps the others)
+  if (s == MAXE_OK && h->tiles) {
+    float ms = 0.f;
+    s = timed([&] { return spmv_tile_launch(h, x, y, nullptr, st); }, &ms);
+    h->tile_use = s == MAXE_OK && ms < 0.95f * best ? 1 : 0;
   }
   // SpMM path for wide right-hand sides, timed at k = 16 when the scratch is modest
   const int64_t k = 16;

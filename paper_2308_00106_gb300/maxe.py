@@ -125,6 +125,7 @@ def load(build_if_missing: bool = False) -> ctypes.CDLL:
             "maxe_handle_tuning": [P, ctypes.POINTER(I32)],
             "maxe_nnz_entropy": [P, I32, I32, ctypes.c_double, ctypes.POINTER(ctypes.c_double), P, P, P],
             "maxe_spmv": [P, P, P, U32, P],
+            "maxe_spmv_tiles": [P, P, P, U32, P],
             "maxe_spmv_host": [P, P, P, P, P, U32, P],
             "maxe_spmm": [P, I32, P, I64, P, I64, U32, P],
             "maxe_power_iteration": [P, P, I32, P, ctypes.POINTER(ctypes.c_double), P],
@@ -264,6 +265,10 @@ class Handle:
         """True when the rows SpMM kernel prefetches each lane group's next X rows (autotuned)."""
         return bool(self._tuning() & 0x40000)
 
+    def spmv_tiles(self) -> bool:
+        """True when SpMV stages the gathered x of a tile of rows in shared memory (kept by the autotuner)."""
+        return bool(self._tuning() & 0x80000)
+
     def xslice_ahead(self) -> int:
         """L2 prefetch distance (entries) of the x-sliced SpMV's entry stream (0: none)."""
         return 512 * ((self._tuning() >> 15) & 7)
@@ -381,6 +386,19 @@ def maxe_spmv(h: Handle, x: torch.Tensor, y: torch.Tensor | None = None, permute
     _dev(y, h.vec_dtype, "y")
     _check(load().maxe_spmv(ctypes.c_void_p(h.ptr), _ptr(x), _ptr(y), MAXE_VEC_PERMUTED if permuted else 0,
                             ctypes.c_void_p(_stream(stream))), "maxe_spmv")
+    return y
+
+
+def maxe_spmv_tiles(h: Handle, x: torch.Tensor, y: torch.Tensor | None = None, permuted: bool = False, stream=None):
+    """y = A x as maxe_spmv, by the staged-tile kernel; needs a handle made with autotune=True."""
+    _dev(x, h.vec_dtype, "x")
+    if x.numel() != h.cols:
+        raise ValueError("x has the wrong length")
+    if y is None:
+        y = torch.empty(h.rows, dtype=h.vec_dtype, device="cuda")
+    _dev(y, h.vec_dtype, "y")
+    _check(load().maxe_spmv_tiles(ctypes.c_void_p(h.ptr), _ptr(x), _ptr(y), MAXE_VEC_PERMUTED if permuted else 0,
+                                  ctypes.c_void_p(_stream(stream))), "maxe_spmv_tiles")
     return y
 
 
