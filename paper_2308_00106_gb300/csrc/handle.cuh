@@ -106,8 +106,10 @@ constexpr int64_t kDefaultBatchTask = 2048;  // entries per warp task of the def
 maxe_status batch_plan(maxe_handle* h, int64_t H, int it16, cudaStream_t st, int lc, int bps = 0);
 maxe_status batch_plan_default(maxe_handle* h, cudaStream_t st);
 
-// spmm_rows.cu: Y = A' X with one row per group of lanes (short rows), when X
-// and Y are 16-byte aligned with whole 16-byte pieces per row.
+// spmm_rows.cu: Y = A' X with one row per group of lanes (short rows).
+// spmm_rows_any: what the launch needs whatever X and Y; spmm_rows_ready: X
+// and Y are also 16-byte aligned with whole 16-byte pieces per row.
+bool spmm_rows_any(const maxe_handle* h, int64_t ldx);
 bool spmm_rows_ready(const maxe_handle* h, int32_t k, const void* X, int64_t ldx, const void* Y, int64_t ldy);
 maxe_status spmm_rows_launch(const maxe_handle* h, int32_t k, const void* X, int64_t ldx, void* Y, int64_t ldy,
                              const int32_t* yperm, cudaStream_t st);

@@ -31,8 +31,14 @@
 // Rows are never split, so each Y row is one group's sum in entry order:
 // deterministic, but a long row holds its group (and its warp) -- the autotuner
 // keeps this path only for matrices where it is faster.  Requires 16-byte
-// aligned X, Y, column and value arrays, with ldx and ldy multiples of VC and
-// ldx rows under 2 GiB.
+// aligned column and value arrays and rows of X under 2 GiB.
+//
+// X or Y rows that are not whole 16-byte pieces (an odd k in contiguous
+// tensors) take a variant whose lanes load 16, 8 or 4 (FP64: 16 or 8) bytes,
+// as X's alignment allows, with up to 32 lanes to a row, and store Y column
+// by column: an X row is still read by one load of the group.  Poisson rows of
+// 20, 100,003 rows, FP32, k = 7 contiguous: 58 us in seven column passes, 21 us
+// here (k = 31: 236 -> 42 us; FP64, k = 7: 131 -> 69 us).
 #include "spmm_rows.cuh"
 
 namespace maxe {
@@ -48,6 +54,7 @@ struct RowsParams {
   RowsOperand op;
   const int32_t* wrow;
   int32_t nW, Q;
+  int32_t G;   // lanes per row, where the kernel has none of its own
   int64_t NG;  // warps of the grid: warp g takes parts g, g + NG, g + 2 NG, ...
 };
 
@@ -74,9 +81,11 @@ __device__ __forceinline__ bool next_start(const RowsParams& p, int32_t* r, int6
   return true;
 }
 
-template <typename VT, int G>
+// GC: lanes per row (0: p.G, a power of two); VC, YVEC: see rows_chunk.
+template <typename VT, int GC, int VC, bool YVEC>
 __global__ void __launch_bounds__(kRowsThreads) spmm_rows_kernel(const RowsParams p) {
   extern __shared__ __align__(16) unsigned char rows_smem[];
+  const int G = GC ? GC : p.G;
   const int lane = threadIdx.x & 31, sub = lane % G, grp = lane / G;
   RowsStage<VT>* s = reinterpret_cast<RowsStage<VT>*>(rows_smem) + (threadIdx.x >> 5);
   // The warp's chunks, part after part, as one sequence: chunk i is multiplied
@@ -105,7 +114,7 @@ __global__ void __launch_bounds__(kRowsThreads) spmm_rows_kernel(const RowsParam
       more2 = next_start(p, &r2, &P2, &b2);
       if (more2) load_rp(p.op.rowptr, r2, b2, lane, &pa, &pb);
     }
-    rows_chunk<VT>(s, buf, p.op, G, 32 / G, grp, sub);
+    rows_chunk<VT, VC, YVEC>(s, buf, p.op, G, 32 / G, grp, sub);
     __syncwarp();
     if (!more) break;
     r1 = r2;
@@ -116,7 +125,7 @@ __global__ void __launch_bounds__(kRowsThreads) spmm_rows_kernel(const RowsParam
   }
 }
 
-template <typename VT, int G>
+template <typename VT, int G, int VC = RowsT<VT>::VC, bool YVEC = true>
 maxe_status launch_rows_g(RowsParams p, int sms, cudaStream_t st) {
   static PerDeviceOnce once;
   static int blocks_per_sm[64];
@@ -124,10 +133,10 @@ maxe_status launch_rows_g(RowsParams p, int sms, cudaStream_t st) {
   int dev = 0;
   MAXE_CUDA_TRY(cudaGetDevice(&dev));
   MAXE_TRY(once.run([dev] {
-    MAXE_CUDA_TRY(cudaFuncSetAttribute(spmm_rows_kernel<VT, G>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    MAXE_CUDA_TRY(cudaFuncSetAttribute(spmm_rows_kernel<VT, G, VC, YVEC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        static_cast<int>(smem)));
     int b = 0;
-    MAXE_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, spmm_rows_kernel<VT, G>, kRowsThreads, smem));
+    MAXE_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, spmm_rows_kernel<VT, G, VC, YVEC>, kRowsThreads, smem));
     blocks_per_sm[dev] = std::max(b, 1);
     return MAXE_OK;
   }));
@@ -135,29 +144,48 @@ maxe_status launch_rows_g(RowsParams p, int sms, cudaStream_t st) {
   const int64_t parts = static_cast<int64_t>(p.nW) * p.Q;
   p.NG = std::max<int64_t>(1, std::min<int64_t>(parts, static_cast<int64_t>(sms) * blocks_per_sm[dev] * kRowsWarps));
   const unsigned grid = static_cast<unsigned>(ceil_div(p.NG, kRowsWarps));
-  spmm_rows_kernel<VT, G><<<grid, kRowsThreads, smem, st>>>(p);
+  spmm_rows_kernel<VT, G, VC, YVEC><<<grid, kRowsThreads, smem, st>>>(p);
   MAXE_CUDA_TRY(cudaGetLastError());
   return MAXE_OK;
 }
 
 template <typename VT>
-maxe_status launch_rows(const RowsParams& p, int sms, cudaStream_t st) {
-  switch (rows_group<VT>(p.op.k)) {
-    case 1: return launch_rows_g<VT, 1>(p, sms, st);
-    case 2: return launch_rows_g<VT, 2>(p, sms, st);
-    case 4: return launch_rows_g<VT, 4>(p, sms, st);
-    default: return launch_rows_g<VT, 8>(p, sms, st);
+maxe_status launch_rows(RowsParams p, int sms, cudaStream_t st) {
+  using AT = typename RowsT<VT>::AT;
+  constexpr int VC = RowsT<VT>::VC;
+  // columns per load that X's rows allow: 16 bytes, 8 (FP32) or one column
+  auto whole = [](const void* q, int64_t ld, int vc) {
+    return ld % vc == 0 && reinterpret_cast<uintptr_t>(q) % (vc * sizeof(AT)) == 0;
+  };
+  if (whole(p.op.X, p.op.ldx, VC) && whole(p.op.Y, p.op.ldy, VC)) {
+    switch (rows_group<VT>(p.op.k)) {
+      case 1: return launch_rows_g<VT, 1>(p, sms, st);
+      case 2: return launch_rows_g<VT, 2>(p, sms, st);
+      case 4: return launch_rows_g<VT, 4>(p, sms, st);
+      default: return launch_rows_g<VT, 8>(p, sms, st);
+    }
   }
+  const int vc = whole(p.op.X, p.op.ldx, VC) ? VC : (whole(p.op.X, p.op.ldx, 2) ? 2 : 1);
+  p.G = 1;  // a lane per piece of the row, at most 32 (more pieces: passes)
+  while (p.G < 32 && p.G * vc < p.op.k) p.G *= 2;
+  if (vc == VC) return launch_rows_g<VT, 0, VC, false>(p, sms, st);
+  if constexpr (VC == 4)
+    if (vc == 2) return launch_rows_g<VT, 0, 2, false>(p, sms, st);
+  return launch_rows_g<VT, 0, 1, false>(p, sms, st);
 }
 
 }  // namespace
 
+bool spmm_rows_any(const maxe_handle* h, int64_t ldx) {
+  const int64_t eb = h->dtype == MAXE_F64 ? 8 : 4;
+  return ldx * eb < (int64_t(1) << 31) &&
+         ((reinterpret_cast<uintptr_t>(h->col) | reinterpret_cast<uintptr_t>(h->val)) & 15u) == 0;
+}
+
 bool spmm_rows_ready(const maxe_handle* h, int32_t k, const void* X, int64_t ldx, const void* Y, int64_t ldy) {
   const int vc = h->dtype == MAXE_F64 ? 2 : 4;
   auto a16 = [](const void* q) { return (reinterpret_cast<uintptr_t>(q) & 15u) == 0; };
-  const int64_t eb = h->dtype == MAXE_F64 ? 8 : 4;
-  return k >= 1 && ldx % vc == 0 && ldy % vc == 0 && ldx * eb < (int64_t(1) << 31) && a16(X) && a16(Y) &&
-         a16(h->col) && a16(h->val);
+  return k >= 1 && ldx % vc == 0 && ldy % vc == 0 && a16(X) && a16(Y) && spmm_rows_any(h, ldx);
 }
 
 maxe_status spmm_rows_launch(const maxe_handle* h, int32_t k, const void* X, int64_t ldx, void* Y, int64_t ldy,

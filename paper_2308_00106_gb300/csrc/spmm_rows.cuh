@@ -33,23 +33,44 @@ struct RowsT;
 template <>
 struct RowsT<float> {
   using AT = float;
-  using V = float4;
-  static constexpr int VC = 4;
+  static constexpr int VC = 4;  // columns of a 16-byte piece
   static __device__ __forceinline__ float acc(float v) { return v; }
 };
 template <>
 struct RowsT<uint16_t> {
   using AT = float;
-  using V = float4;
   static constexpr int VC = 4;
   static __device__ __forceinline__ float acc(uint16_t v) { return __uint_as_float(static_cast<uint32_t>(v) << 16); }
 };
 template <>
 struct RowsT<double> {
   using AT = double;
-  using V = double2;
   static constexpr int VC = 2;
   static __device__ __forceinline__ double acc(double v) { return v; }
+};
+
+// A lane's piece of VC columns.
+template <typename AT, int VC>
+struct RowsPiece;
+template <>
+struct RowsPiece<float, 4> {
+  using V = float4;
+};
+template <>
+struct RowsPiece<float, 2> {
+  using V = float2;
+};
+template <>
+struct RowsPiece<float, 1> {
+  using V = float;
+};
+template <>
+struct RowsPiece<double, 2> {
+  using V = double2;
+};
+template <>
+struct RowsPiece<double, 1> {
+  using V = double;
 };
 
 __device__ __forceinline__ void fma_vec(float4& acc, float a, const float4& x) {
@@ -58,6 +79,12 @@ __device__ __forceinline__ void fma_vec(float4& acc, float a, const float4& x) {
   acc.z = fmaf(a, x.z, acc.z);
   acc.w = fmaf(a, x.w, acc.w);
 }
+__device__ __forceinline__ void fma_vec(float2& acc, float a, const float2& x) {
+  acc.x = fmaf(a, x.x, acc.x);
+  acc.y = fmaf(a, x.y, acc.y);
+}
+__device__ __forceinline__ void fma_vec(float& acc, float a, float x) { acc = fmaf(a, x, acc); }
+__device__ __forceinline__ void fma_vec(double& acc, double a, double x) { acc = fma(a, x, acc); }
 __device__ __forceinline__ void fma_vec(double2& acc, double a, const double2& x) {
   acc.x = fma(a, x.x, acc.x);
   acc.y = fma(a, x.y, acc.y);
@@ -72,6 +99,12 @@ __device__ __forceinline__ void add_vec(double2& a, const double2& b) {
   a.x += b.x;
   a.y += b.y;
 }
+__device__ __forceinline__ void add_vec(float2& a, const float2& b) {
+  a.x += b.x;
+  a.y += b.y;
+}
+__device__ __forceinline__ void add_vec(float& a, float b) { a += b; }
+__device__ __forceinline__ void add_vec(double& a, double b) { a += b; }
 // Y piece of a row: all VC columns, or the first `left` of them (the row's last piece)
 __device__ __forceinline__ void store_piece(float4* y, const float4& v, int left) {
   if (left >= 4) {
@@ -90,6 +123,17 @@ __device__ __forceinline__ void store_piece(double2* y, const double2& v, int le
   }
   reinterpret_cast<double*>(y)[0] = v.x;
 }
+// Y rows that are not 16-byte aligned: column by column
+template <typename AT, typename V>
+__device__ __forceinline__ void store_columns(AT* y, const V& v, int left) {
+  const AT* f = reinterpret_cast<const AT*>(&v);
+#pragma unroll
+  for (int c = 0; c < static_cast<int>(sizeof(V) / sizeof(AT)); ++c)
+    if (c < left) y[c] = f[c];
+}
+__device__ __forceinline__ void zero(float2& v) { v = make_float2(0.f, 0.f); }
+__device__ __forceinline__ void zero(float& v) { v = 0.f; }
+__device__ __forceinline__ void zero(double& v) { v = 0.0; }
 __device__ __forceinline__ void zero(float4& v) { v = make_float4(0.f, 0.f, 0.f, 0.f); }
 __device__ __forceinline__ void zero(double2& v) { v = make_double2(0.0, 0.0); }
 
@@ -173,15 +217,15 @@ __device__ __forceinline__ int32_t stage_chunk(RowsStage<VT>* s, int buf, const 
 }
 
 // Multiplies the rows of chunk buffer `buf` and writes their Y pieces: lane
-// `sub` of group `grp` (G lanes per group, GPW = 32 / G groups per warp).
-template <typename VT>
+// `sub` of group `grp` (G lanes per group, GPW = 32 / G groups per warp), each
+// lane VC columns.  YVEC: Y rows are 16-byte aligned and VC is a whole 16 bytes.
+// A row's sum does not depend on VC, G or YVEC.
+template <typename VT, int VC = RowsT<VT>::VC, bool YVEC = true>
 __device__ __forceinline__ void rows_chunk(const RowsStage<VT>* s, int buf, const RowsOperand& p, int G, int GPW,
                                            int grp, int sub) {
   using T = RowsT<VT>;
-  using V = typename T::V;
   using AT = typename T::AT;
-  constexpr int VC = T::VC;
-  V* Y = static_cast<V*>(p.Y);
+  using V = typename RowsPiece<AT, VC>::V;
   const int32_t ldx_bytes = static_cast<int32_t>(p.ldx * static_cast<int64_t>(sizeof(AT)));  // < 2^31 (checked)
   const int64_t ldyv = p.ldy / VC;
   const int kv = (p.k + VC - 1) / VC;
@@ -205,7 +249,7 @@ __device__ __forceinline__ void rows_chunk(const RowsStage<VT>* s, int buf, cons
     }
     for (int c = sub; c < kv; c += G) {
       // X piece c of row COL: xc + COL * ldx_bytes (one wide multiply-add per entry)
-      const char* xc = static_cast<const char*>(p.X) + 16 * c;
+      const char* xc = static_cast<const char*>(p.X) + static_cast<int>(sizeof(V)) * c;
       V part[kRowsParts];
 #pragma unroll
       for (int u = 0; u < kRowsParts; ++u) zero(part[u]);
@@ -244,7 +288,10 @@ __device__ __forceinline__ void rows_chunk(const RowsStage<VT>* s, int buf, cons
       add_vec(part[0], part[1]);
       add_vec(part[2], part[3]);
       add_vec(part[0], part[2]);
-      store_piece(Y + yr * ldyv + c, part[0], p.k - c * VC);
+      if constexpr (YVEC)
+        store_piece(static_cast<V*>(p.Y) + yr * ldyv + c, part[0], p.k - c * VC);
+      else
+        store_columns(static_cast<AT*>(p.Y) + yr * p.ldy + c * VC, part[0], p.k - c * VC);
     }
   }
 }

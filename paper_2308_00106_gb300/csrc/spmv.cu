@@ -184,7 +184,7 @@ maxe_status spmm_launch(const maxe_handle* h, int32_t k, const void* X, int64_t 
   const bool unit = k == 1 && ldx == 1 && ldy == 1;
   if (unit && variant == -1 && lc < 0 && h->tile_use) return spmv_tile_launch(h, X, Y, yperm, st);
   if (unit && variant < 0 && lc < 0 && xslice_ready(h, X)) return xslice_launch(h, X, Y, yperm, st);
-  if (k > 1 && variant < 0 && lc < 0 && h->spmm_rows && spmm_rows_ready(h, k, X, ldx, Y, ldy))
+  if (k > 1 && variant < 0 && lc < 0 && h->spmm_rows && spmm_rows_any(h, ldx))
     return spmm_rows_launch(h, k, X, ldx, Y, ldy, yperm, st);
   const int it = (unit && variant < 0) ? h->spmv_items16 : (variant > 0 ? 1 : 0);
   if (it == 1 && !unit) return MAXE_ERR_UNSUPPORTED;
