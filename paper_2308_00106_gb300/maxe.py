@@ -105,6 +105,8 @@ def lib_path() -> str:
 def load(build_if_missing: bool = False) -> ctypes.CDLL:
     """Load libmaxe.so; raises if it has not been built (no fallback path)."""
     global _lib
+    if _lib is not None:  # once set it stays
+        return _lib
     with _lock:
         if _lib is not None:
             return _lib
@@ -176,7 +178,7 @@ def _check(s: int, what: str):
 
 def _stream(stream=None) -> int:
     if stream is None:
-        stream = torch.cuda.current_stream()
+        return torch.cuda.current_stream().cuda_stream
     return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
 
@@ -191,7 +193,7 @@ def _dev(t: torch.Tensor, dtype, name: str) -> torch.Tensor:
 
 
 def _ptr(t: torch.Tensor | None):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 class _DevArray:
@@ -229,7 +231,7 @@ class Handle:
         """(rowptr, col, val, rperm, cperm) as zero-copy torch views of the handle's arrays."""
         v = _Csr()
         rp, cp = ctypes.c_void_p(), ctypes.c_void_p()
-        _check(load().maxe_handle_csr(ctypes.c_void_p(self.ptr), ctypes.byref(v), ctypes.byref(rp), ctypes.byref(cp)),
+        _check(load().maxe_handle_csr(self.ptr, ctypes.byref(v), ctypes.byref(rp), ctypes.byref(cp)),
                "maxe_handle_csr")
         return (_view(v.rowptr, self.rows + 1, torch.int32), _view(v.col, self.nnz, torch.int32),
                 _view(v.val, self.nnz, VAL_TORCH[self.dtype]), _view(rp.value, self.rows, torch.int32),
@@ -238,7 +240,7 @@ class Handle:
     def coo_rows(self):
         """COO row index of every entry (zero-copy view), for handles made with coo=True."""
         r = ctypes.c_void_p()
-        _check(load().maxe_handle_coo(ctypes.c_void_p(self.ptr), ctypes.byref(r)), "maxe_handle_coo")
+        _check(load().maxe_handle_coo(self.ptr, ctypes.byref(r)), "maxe_handle_coo")
         return _view(r.value, self.nnz, torch.int32)
 
     def items_per_lane(self) -> int:
@@ -283,12 +285,12 @@ class Handle:
 
     def _tuning(self) -> int:
         v = ctypes.c_int32()
-        _check(load().maxe_handle_tuning(ctypes.c_void_p(self.ptr), ctypes.byref(v)), "maxe_handle_tuning")
+        _check(load().maxe_handle_tuning(self.ptr, ctypes.byref(v)), "maxe_handle_tuning")
         return v.value
 
     def close(self):
         if self.ptr:
-            load().maxe_handle_destroy(ctypes.c_void_p(self.ptr))
+            load().maxe_handle_destroy(self.ptr)
             self.ptr = 0
 
     def __del__(self):
@@ -306,7 +308,7 @@ def maxe_build_permutation(seed: int, n: int, tag: int, perm: torch.Tensor | Non
         perm = torch.empty(n, dtype=torch.int32, device="cuda")
     _dev(perm, torch.int32, "perm")
     _check(load().maxe_build_permutation(ctypes.c_uint64(seed & (2**64 - 1)), n, tag, _ptr(perm),
-                                         ctypes.byref(_ALLOC), ctypes.c_void_p(_stream(stream))),
+                                         ctypes.byref(_ALLOC), _stream(stream)),
            "maxe_build_permutation")
     return perm
 
@@ -314,7 +316,7 @@ def maxe_build_permutation(seed: int, n: int, tag: int, perm: torch.Tensor | Non
 def maxe_invert_permutation(perm: torch.Tensor, stream=None):
     _dev(perm, torch.int32, "perm")
     inv = torch.empty_like(perm)
-    _check(load().maxe_invert_permutation(_ptr(perm), perm.numel(), _ptr(inv), ctypes.c_void_p(_stream(stream))),
+    _check(load().maxe_invert_permutation(_ptr(perm), perm.numel(), _ptr(inv), _stream(stream)),
            "maxe_invert_permutation")
     return inv
 
@@ -324,7 +326,7 @@ def maxe_permute_gather(perm: torch.Tensor, x: torch.Tensor, stream=None):
     _dev(perm, torch.int32, "perm")
     out = torch.empty(perm.numel(), dtype=x.dtype, device="cuda")
     _check(load().maxe_permute_gather(_ptr(perm), perm.numel(), x.element_size(), _ptr(x), _ptr(out),
-                                      ctypes.c_void_p(_stream(stream))), "maxe_permute_gather")
+                                      _stream(stream)), "maxe_permute_gather")
     return out
 
 
@@ -333,7 +335,7 @@ def maxe_permute_scatter(perm: torch.Tensor, y: torch.Tensor, stream=None):
     _dev(perm, torch.int32, "perm")
     out = torch.empty(perm.numel(), dtype=y.dtype, device="cuda")
     _check(load().maxe_permute_scatter(_ptr(perm), perm.numel(), y.element_size(), _ptr(y), _ptr(out),
-                                       ctypes.c_void_p(_stream(stream))), "maxe_permute_scatter")
+                                       _stream(stream)), "maxe_permute_scatter")
     return out
 
 
@@ -362,7 +364,7 @@ def maxe_permute_csr(rows: int, cols: int, rowptr: torch.Tensor, col: torch.Tens
              | (0 if xs_pairs is None else (MAXE_XS_PAIRS if xs_pairs else MAXE_XS_SINGLE))
              | (MAXE_SPMM_ROWS if spmm_rows else 0) | (MAXE_SPMM_ROWS_PF if spmm_rows_pf else 0))
     _check(load().maxe_permute_csr(ctypes.byref(A), _ptr(rperm), _ptr(cperm), flags,
-                                   ctypes.byref(_ALLOC), ctypes.c_void_p(_stream(stream)), ctypes.byref(out)),
+                                   ctypes.byref(_ALLOC), _stream(stream), ctypes.byref(out)),
            "maxe_permute_csr")
     return Handle(out.value, rows, cols, col.numel(), code, keep=None)
 
@@ -371,8 +373,8 @@ def maxe_nnz_entropy(h: Handle, gr: int, gc: int, base: float = 2.0, counts: boo
     """(H, counts[gr, gc] int64 or None) of the nonzero block-grid histogram (Section 4)."""
     H = ctypes.c_double()
     cnt = torch.empty(gr * gc, dtype=torch.int64, device="cuda") if counts else None
-    _check(load().maxe_nnz_entropy(ctypes.c_void_p(h.ptr), gr, gc, float(base), ctypes.byref(H), _ptr(cnt),
-                                   ctypes.byref(_ALLOC), ctypes.c_void_p(_stream(stream))), "maxe_nnz_entropy")
+    _check(load().maxe_nnz_entropy(h.ptr, gr, gc, float(base), ctypes.byref(H), _ptr(cnt),
+                                   ctypes.byref(_ALLOC), _stream(stream)), "maxe_nnz_entropy")
     return H.value, (cnt.view(gr, gc) if counts else None)
 
 
@@ -384,8 +386,8 @@ def maxe_spmv(h: Handle, x: torch.Tensor, y: torch.Tensor | None = None, permute
     if y is None:
         y = torch.empty(h.rows, dtype=h.vec_dtype, device="cuda")
     _dev(y, h.vec_dtype, "y")
-    _check(load().maxe_spmv(ctypes.c_void_p(h.ptr), _ptr(x), _ptr(y), MAXE_VEC_PERMUTED if permuted else 0,
-                            ctypes.c_void_p(_stream(stream))), "maxe_spmv")
+    _check(load().maxe_spmv(h.ptr, _ptr(x), _ptr(y), MAXE_VEC_PERMUTED if permuted else 0,
+                            _stream(stream)), "maxe_spmv")
     return y
 
 
@@ -397,8 +399,8 @@ def maxe_spmv_tiles(h: Handle, x: torch.Tensor, y: torch.Tensor | None = None, p
     if y is None:
         y = torch.empty(h.rows, dtype=h.vec_dtype, device="cuda")
     _dev(y, h.vec_dtype, "y")
-    _check(load().maxe_spmv_tiles(ctypes.c_void_p(h.ptr), _ptr(x), _ptr(y), MAXE_VEC_PERMUTED if permuted else 0,
-                                  ctypes.c_void_p(_stream(stream))), "maxe_spmv_tiles")
+    _check(load().maxe_spmv_tiles(h.ptr, _ptr(x), _ptr(y), MAXE_VEC_PERMUTED if permuted else 0,
+                                  _stream(stream)), "maxe_spmv_tiles")
     return y
 
 
@@ -424,8 +426,8 @@ def maxe_spmv_host(h: Handle, x_host: torch.Tensor, y_host: torch.Tensor, x_dev:
     _dev(y_dev, h.vec_dtype, "y_dev")
     if x_dev.numel() != h.cols or y_dev.numel() != h.rows:
         raise ValueError("x_dev / y_dev have the wrong length")
-    _check(load().maxe_spmv_host(ctypes.c_void_p(h.ptr), _ptr(x_host), _ptr(y_host), _ptr(x_dev), _ptr(y_dev),
-                                 MAXE_VEC_PERMUTED if permuted else 0, ctypes.c_void_p(_stream(stream))),
+    _check(load().maxe_spmv_host(h.ptr, _ptr(x_host), _ptr(y_host), _ptr(x_dev), _ptr(y_dev),
+                                 MAXE_VEC_PERMUTED if permuted else 0, _stream(stream)),
            "maxe_spmv_host")
     return y_host
 
@@ -438,8 +440,8 @@ def maxe_coo_spmv(h: Handle, x: torch.Tensor, y: torch.Tensor | None = None, per
     if y is None:
         y = torch.empty(h.rows, dtype=h.vec_dtype, device="cuda")
     _dev(y, h.vec_dtype, "y")
-    _check(load().maxe_coo_spmv(ctypes.c_void_p(h.ptr), _ptr(x), _ptr(y), MAXE_VEC_PERMUTED if permuted else 0,
-                                ctypes.c_void_p(_stream(stream))), "maxe_coo_spmv")
+    _check(load().maxe_coo_spmv(h.ptr, _ptr(x), _ptr(y), MAXE_VEC_PERMUTED if permuted else 0,
+                                _stream(stream)), "maxe_coo_spmv")
     return y
 
 
@@ -454,8 +456,8 @@ def maxe_spmm(h: Handle, X: torch.Tensor, Y: torch.Tensor | None = None, permute
         Y = torch.empty(h.rows, k, dtype=h.vec_dtype, device="cuda")
     if Y.stride(1) != 1 or Y.shape != (h.rows, k):
         raise ValueError("Y must be (rows, k) with unit column stride")
-    _check(load().maxe_spmm(ctypes.c_void_p(h.ptr), k, _ptr(X), X.stride(0), _ptr(Y), Y.stride(0),
-                            MAXE_VEC_PERMUTED if permuted else 0, ctypes.c_void_p(_stream(stream))), "maxe_spmm")
+    _check(load().maxe_spmm(h.ptr, k, _ptr(X), X.stride(0), _ptr(Y), Y.stride(0),
+                            MAXE_VEC_PERMUTED if permuted else 0, _stream(stream)), "maxe_spmm")
     return Y
 
 
@@ -467,17 +469,17 @@ def maxe_power_iteration(h: Handle, v0: torch.Tensor, steps: int, stream=None, h
     lam = ctypes.c_double()
     if history:
         hist = (ctypes.c_double * max(steps, 1))()
-        _check(load().maxe_power_iteration_history(ctypes.c_void_p(h.ptr), _ptr(v0), steps, _ptr(v),
-                                                   ctypes.byref(lam), hist, ctypes.c_void_p(_stream(stream))),
+        _check(load().maxe_power_iteration_history(h.ptr, _ptr(v0), steps, _ptr(v),
+                                                   ctypes.byref(lam), hist, _stream(stream)),
                "maxe_power_iteration_history")
         return lam.value, v, np.array(hist[:steps], dtype=np.float64)
-    _check(load().maxe_power_iteration(ctypes.c_void_p(h.ptr), _ptr(v0), steps, _ptr(v), ctypes.byref(lam),
-                                       ctypes.c_void_p(_stream(stream))), "maxe_power_iteration")
+    _check(load().maxe_power_iteration(h.ptr, _ptr(v0), steps, _ptr(v), ctypes.byref(lam),
+                                       _stream(stream)), "maxe_power_iteration")
     return lam.value, v
 
 
 def maxe_device_status(stream=None) -> int:
-    return load().maxe_device_status(ctypes.c_void_p(_stream(stream)))
+    return load().maxe_device_status(_stream(stream))
 
 
 def maxe_set_wait_limit_ns(ns: int):
@@ -487,7 +489,7 @@ def maxe_set_wait_limit_ns(ns: int):
 
 def maxe_selftest_wait(stream=None):
     """Launch a wait on a flag nothing sets; it runs out after the wait limit."""
-    _check(load().maxe_selftest_wait(ctypes.c_void_p(_stream(stream))), "maxe_selftest_wait")
+    _check(load().maxe_selftest_wait(_stream(stream)), "maxe_selftest_wait")
 
 
 def maxe_version() -> str:
@@ -511,7 +513,7 @@ class Batch:
 
     def __init__(self, capacity: int, stream=None):
         out = ctypes.c_void_p()
-        _check(load().maxe_batch_create(capacity, ctypes.byref(_ALLOC), ctypes.c_void_p(_stream(stream)),
+        _check(load().maxe_batch_create(capacity, ctypes.byref(_ALLOC), _stream(stream),
                                         ctypes.byref(out)), "maxe_batch_create")
         self.ptr = out.value
         self._keep = []
@@ -530,15 +532,15 @@ class Batch:
             arr[i] = _BatchItem(h.ptr, k, X.data_ptr(), X.stride(0), Y.data_ptr(), Y.stride(0),
                                 MAXE_BATCH_SCATTER_Y if scatter else 0)
             keep += [h, X, Y]
-        _check(load().maxe_batch_set(ctypes.c_void_p(self.ptr), arr, len(items)), "maxe_batch_set")
+        _check(load().maxe_batch_set(self.ptr, arr, len(items)), "maxe_batch_set")
         self._keep = keep
 
     def run(self, stream=None):
-        _check(load().maxe_batch_run(ctypes.c_void_p(self.ptr), ctypes.c_void_p(_stream(stream))), "maxe_batch_run")
+        _check(load().maxe_batch_run(self.ptr, _stream(stream)), "maxe_batch_run")
 
     def close(self):
         if self.ptr:
-            load().maxe_batch_destroy(ctypes.c_void_p(self.ptr))
+            load().maxe_batch_destroy(self.ptr)
             self.ptr = 0
 
     def __del__(self):
@@ -549,13 +551,13 @@ class Batch:
 
 
 def maxe_batch_tune(h: Handle, k: int, stream=None):
-    _check(load().maxe_batch_tune(ctypes.c_void_p(h.ptr), k, ctypes.c_void_p(_stream(stream))), "maxe_batch_tune")
+    _check(load().maxe_batch_tune(h.ptr, k, _stream(stream)), "maxe_batch_tune")
 
 
 def maxe_batch_plan_info(h: Handle):
     """(entries per warp task, tasks, entries per lane) of the handle's batch plan."""
     H, t, it = ctypes.c_int64(), ctypes.c_int32(), ctypes.c_int32()
-    _check(load().maxe_batch_plan_info(ctypes.c_void_p(h.ptr), ctypes.byref(H), ctypes.byref(t), ctypes.byref(it)),
+    _check(load().maxe_batch_plan_info(h.ptr, ctypes.byref(H), ctypes.byref(t), ctypes.byref(it)),
            "maxe_batch_plan_info")
     return H.value, t.value, it.value
 
@@ -563,21 +565,21 @@ def maxe_batch_plan_info(h: Handle):
 def maxe_batch_plan_shape(h: Handle) -> int:
     """CTAs per SM the handle's batch plan asks of a launch (0: as many as fit)."""
     v = ctypes.c_int32()
-    _check(load().maxe_batch_plan_shape(ctypes.c_void_p(h.ptr), ctypes.byref(v)), "maxe_batch_plan_shape")
+    _check(load().maxe_batch_plan_shape(h.ptr, ctypes.byref(v)), "maxe_batch_plan_shape")
     return v.value
 
 
 def maxe_vec_norm_gather(Q: torch.Tensor | None, w: torch.Tensor, u: torch.Tensor, scratch: torch.Tensor, stream=None):
     """u[j] = w[Q[j]] / ||w||_2 (FP64 norm); scratch: >= 514 float64 on the device."""
     _check(load().maxe_vec_norm_gather(_ptr(Q), w.numel(), w.element_size(), _ptr(w), _ptr(u), _ptr(scratch),
-                                       ctypes.c_void_p(_stream(stream))), "maxe_vec_norm_gather")
+                                       _stream(stream)), "maxe_vec_norm_gather")
 
 
 def maxe_vec_dot_gather(Q: torch.Tensor | None, u: torch.Tensor, w: torch.Tensor, scratch: torch.Tensor,
                         out: torch.Tensor, stream=None):
     """out[0] = sum_j u[j] * w[Q[j]] (FP64)."""
     _check(load().maxe_vec_dot_gather(_ptr(Q), u.numel(), u.element_size(), _ptr(u), _ptr(w), _ptr(scratch),
-                                      _ptr(out), ctypes.c_void_p(_stream(stream))), "maxe_vec_dot_gather")
+                                      _ptr(out), _stream(stream)), "maxe_vec_dot_gather")
 
 
 def maxe_entropy_levels(counts: torch.Tensor, L: int, base: float = 2.0, stream=None) -> torch.Tensor:
@@ -586,7 +588,7 @@ def maxe_entropy_levels(counts: torch.Tensor, L: int, base: float = 2.0, stream=
     gr, gc = counts.shape
     out = torch.empty(L * L, dtype=torch.float64, device="cuda")
     _check(load().maxe_entropy_levels(_ptr(counts), gr, gc, L, float(base), _ptr(out),
-                                      ctypes.c_void_p(_stream(stream))), "maxe_entropy_levels")
+                                      _stream(stream)), "maxe_entropy_levels")
     return out.view(L, L)
 
 
@@ -601,7 +603,7 @@ def maxe_nnz_histogram(A, axis: int, stream=None) -> torch.Tensor:
     _dev(A.rowptr, torch.int32, "rowptr")
     hist = torch.empty(A.rows if axis == 0 else A.cols, dtype=torch.int32, device="cuda")
     s = _csr_struct(A)
-    _check(load().maxe_nnz_histogram(ctypes.byref(s), int(axis), _ptr(hist), ctypes.c_void_p(_stream(stream))),
+    _check(load().maxe_nnz_histogram(ctypes.byref(s), int(axis), _ptr(hist), _stream(stream)),
            "maxe_nnz_histogram")
     return hist
 
@@ -615,7 +617,7 @@ def maxe_gradient_permutation(hist: torch.Tensor, seed: int, tag: int, stream=No
     perm = torch.empty(n, dtype=torch.int32, device="cuda")
     pivot = torch.empty(1, dtype=torch.int32, device="cuda")
     _check(load().maxe_gradient_permutation(_ptr(hist), n, ctypes.c_uint64(seed & (2**64 - 1)), tag, _ptr(perm),
-                                            _ptr(pivot), ctypes.byref(_ALLOC), ctypes.c_void_p(_stream(stream))),
+                                            _ptr(pivot), ctypes.byref(_ALLOC), _stream(stream)),
            "maxe_gradient_permutation")
     return perm, pivot
 

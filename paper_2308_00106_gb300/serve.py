@@ -21,7 +21,11 @@ about two steps per stream, so admitting interleaves with launching); each
 batch step takes one unit of work (a product) from
 admitted requests that are not already on the GPU, oldest first, up to a byte
 budget of work per step, so requests join and leave between steps and a power
-iteration advances one product per step.  Two CUDA streams, each with its own
+iteration advances one product per step -- or, while no other request waits to
+join, as many as the step's budget holds, in rounds one behind the other on the
+step's stream (a host round trip per product cost more than the product:
+two 20-step iterations on 300k-row matrices took most of a 7.5 ms trace).
+Requests of one product are done after the first round.  Two CUDA streams, each with its own
 batch object, keep two steps in flight, so a step's work overlaps the previous
 one on the device.  Every matrix has a fixed
 batch plan, so a request's result is bit-identical alone and in any mix.
@@ -113,6 +117,7 @@ class Server:
                 self.Q.append(None)
             resident += A.nnz * (4 + A.val.element_size()) + (A.rows + 1) * 4 + (A.rows + A.cols) * 4 * 2
         torch.cuda.synchronize()
+        self.sliced = [h.xslice() for h in self.handles]  # fixed once a handle is made
         self.resident_bytes = resident
         self.mem_cap = mem_cap_bytes
         self.streams = [torch.cuda.Stream() for _ in range(streams)]
@@ -145,7 +150,7 @@ class Server:
             g = self.gen
             g.manual_seed(r.seed)
             if r.kind == "power":
-                u = torch.rand(A.cols, generator=g, device="cuda") * 2 - 1
+                u = torch.empty(A.cols, device="cuda").uniform_(-1, 1, generator=g)
                 r.bufs = {"u": u, "w": torch.empty(A.rows, device="cuda"),
                           "scratch": torch.empty(1024, dtype=torch.float64, device="cuda"),
                           "lam": torch.empty(1, dtype=torch.float64, device="cuda"), "u0": u.clone()}
@@ -153,19 +158,18 @@ class Server:
                 # 16-byte rows for k > 1 (the kernel gathers 4 columns per load); unit
                 # strides for k = 1, which the batched kernel runs in its SpMV class
                 kp = 1 if r.k == 1 else (r.k + 3) // 4 * 4
-                if kp == r.k:
-                    X = torch.rand(A.cols, r.k, generator=g, device="cuda").mul_(2).sub_(1)
-                else:
-                    X = torch.zeros(A.cols, kp, device="cuda")
-                    X[:, :r.k] = torch.rand(A.cols, r.k, generator=g, device="cuda") * 2 - 1
+                X = torch.empty(A.cols, r.k, device="cuda").uniform_(-1, 1, generator=g)
+                if kp != r.k:
+                    X = torch.nn.functional.pad(X, (0, kp - r.k))
                 r.bufs = {"X": X[:, :r.k], "Y": torch.empty(A.rows, kp, device="cuda")[:, :r.k]}
 
     def _launch(self, si: int, reqs):
-        """One step on stream si: the products of `reqs` (single SpMV launches
+        """One round on stream si: the products of `reqs` (single SpMV launches
         where the handle runs the x-sliced form, which one persistent batched
         launch would not use; one batched launch per kernel class for the
         rest), then the power iterations' vector steps."""
         s = self.streams[si]
+        st = s.cuda_stream
         items, singles = [], []
         for r in reqs:
             h = self.handles[r.mat]
@@ -173,26 +177,30 @@ class Server:
                 x, y = r.bufs["u"], r.bufs["w"]
             else:
                 x, y = r.bufs["X"], r.bufs["Y"]
-            if (r.kind == "power" or r.k == 1) and h.xslice():
+            if (r.kind == "power" or r.k == 1) and self.sliced[r.mat]:
                 singles.append((h, x.reshape(-1), y.reshape(-1)))
             else:
                 items.append((h, x, y, False))
-        b = self.batches[si]
-        b.set(items)
-        b.run(stream=s)
+        if items:
+            b = self.batches[si]
+            b.set(items)
+            b.run(stream=st)
         for h, x, y in singles:
-            maxe.maxe_spmv(h, x, y, permuted=True, stream=s)
-        with torch.cuda.stream(s):
-            for r in reqs:
-                if r.kind != "power":
-                    continue
-                if r.units_done < r.steps:  # normalise: u <- Q(w) / ||w||
-                    maxe.maxe_vec_norm_gather(self.Q[r.mat], r.bufs["w"], r.bufs["u"], r.bufs["scratch"], stream=s)
-                else:  # lambda = u . Q(w)
-                    maxe.maxe_vec_dot_gather(self.Q[r.mat], r.bufs["u"], r.bufs["w"], r.bufs["scratch"],
-                                             r.bufs["lam"], stream=s)
+            maxe.maxe_spmv(h, x, y, permuted=True, stream=st)
+        for r in reqs:
+            if r.kind != "power":
+                continue
+            if r.units_done < r.steps:  # normalise: u <- Q(w) / ||w||
+                maxe.maxe_vec_norm_gather(self.Q[r.mat], r.bufs["w"], r.bufs["u"], r.bufs["scratch"], stream=st)
+            else:  # lambda = u . Q(w)
+                maxe.maxe_vec_dot_gather(self.Q[r.mat], r.bufs["u"], r.bufs["w"], r.bufs["scratch"],
+                                         r.bufs["lam"], stream=st)
+        for r in reqs:
+            r.units_done += 1
+
+    def _event(self, si: int):
         ev = torch.cuda.Event()
-        ev.record(s)
+        ev.record(self.streams[si])
         return ev
 
     def _finish(self, r: Request, keep: bool):
@@ -201,17 +209,12 @@ class Server:
                 r.result = (float(r.bufs["lam"].item()), r.bufs["u"].clone(), r.bufs["u0"])
             else:
                 r.result = r.bufs["Y"].contiguous()
-            # The copies above are queued on the current stream, but the buffers
-            # belong to adm_stream: once dropped, the caching allocator may hand
-            # them to the next admission on adm_stream, so that stream must not
-            # run ahead of the copies.
-            self.adm_stream.wait_stream(torch.cuda.current_stream())
         r.bufs = {}
 
     # ------------------------------------------------------------ the loop
     def run(self, trace, keep_results: bool = False, max_wall: float = 600.0, max_items: int | None = None):
         """Serve `trace` (requests sorted by arrival); returns a stats dict.
-        max_items caps the requests per batch step (1 = no batching)."""
+        max_items caps the products per batch step (1 = no batching)."""
         cap_items = self.capacity if max_items is None else max(1, min(max_items, self.capacity))
         trace = sorted(trace, key=lambda r: r.arrival)
         n = len(trace)
@@ -228,6 +231,7 @@ class Server:
         steps = 0
         peak_mem = 0
         max_batch = 0
+        idle = 0  # polls in a row that found nothing to do
         t0 = time.perf_counter()
         while done < n:
             now = time.perf_counter() - t0
@@ -254,8 +258,6 @@ class Server:
                 del inflight[si]
                 tnow = time.perf_counter() - t0
                 for r in reqs:
-                    r.units_done += 1
-                    bytes_done += self.unit_bytes(r)
                     if r.units_done >= r.units:
                         r.t_done = tnow
                         self._finish(r, keep_results)
@@ -264,34 +266,60 @@ class Server:
                     else:
                         ready.append(r)
                         ready_work += self.unit_bytes(r)
+                if keep_results:
+                    # The results' copies are queued on the current stream, but the
+                    # dropped buffers belong to adm_stream: the caching allocator may
+                    # hand them to the next admission on adm_stream, so that stream
+                    # must not run ahead of the copies.
+                    self.adm_stream.wait_stream(torch.cuda.current_stream())
                 progressed = True
             for si in range(len(self.streams)):
                 if si in inflight or not ready:
                     continue
+                # only power iterations, and nobody waits to join: the idle streams
+                # share them, each for several products
+                rounds = not waiting and all(r.kind == "power" for r in ready)
+                most = cap_items
+                if rounds:
+                    most = min(most, -(-len(ready) // (len(self.streams) - len(inflight))))
                 take, work = [], 0
-                while ready and len(take) < cap_items and (not take or work < self.step_bytes):
+                while ready and len(take) < most and (not take or work < self.step_bytes):
                     r = ready.popleft()
                     take.append(r)
                     work += self.unit_bytes(r)
                 ready_work -= work
                 # the first step of a freshly admitted request must see its initialised buffers
                 self.streams[si].wait_stream(self.adm_stream)
-                inflight[si] = (self._launch(si, take), take)
+                self._launch(si, take)
+                bytes_done += work
+                products = len(take)
+                left = [r for r in take if r.units_done < r.units] if rounds else []
+                while left and work < self.step_bytes and products + len(left) <= cap_items:
+                    self._launch(si, left)
+                    more = sum(self.unit_bytes(r) for r in left)
+                    work += more
+                    bytes_done += more
+                    products += len(left)
+                    left = [r for r in left if r.units_done < r.units]
+                inflight[si] = (self._event(si), take)
                 steps += 1
                 max_batch = max(max_batch, len(take))
                 progressed = True
-            if not progressed:
-                time.sleep(20e-6)
+            # yield at first: a sleep of any length takes some 70 us, as long as a step
+            idle = 0 if progressed else idle + 1
+            if idle:
+                time.sleep(0 if idle < 200 else 20e-6)
         wall = time.perf_counter() - t0
         lat = np.array([r.latency for r in trace])
         by = {}
         for kind in ("spmv", "spmm", "power"):
             v = np.array([r.latency for r in trace if r.kind == kind])
             if v.size:
-                by[kind] = {"n": int(v.size), "p50_ms": float(np.percentile(v, 50) * 1e3),
-                            "p99_ms": float(np.percentile(v, 99) * 1e3)}
+                p50, p99 = np.percentile(v, (50, 99)) * 1e3
+                by[kind] = {"n": int(v.size), "p50_ms": float(p50), "p99_ms": float(p99)}
+        p50, p99 = np.percentile(lat, (50, 99)) * 1e3
         return {"requests": n, "wall_s": wall, "req_per_s": n / wall, "gbs": bytes_done / wall / 1e9,
-                "p50_ms": float(np.percentile(lat, 50) * 1e3), "p99_ms": float(np.percentile(lat, 99) * 1e3),
+                "p50_ms": float(p50), "p99_ms": float(p99),
                 "by_kind": by, "batch_steps": steps, "max_batch": max_batch, "peak_request_bytes": peak_mem,
                 "resident_bytes": self.resident_bytes}
 
