@@ -109,11 +109,12 @@ typedef enum { MAXE_F64 = 0, MAXE_F32 = 1, MAXE_BF16 = 2 } maxe_dtype;
 #define MAXE_XS_PAIRS 0x100u
 #define MAXE_XS_SINGLE 0x200u
 /* Flag of maxe_permute_csr: SpMM (k > 1) with one row per group of lanes --
- * each lane holds 16 bytes of the k columns of X and Y (4 FP32 / 2 FP64), a
- * group walks its row's entries and writes its piece of Y once -- for matrices
- * with short rows, when X and Y are 16-byte aligned and ldx, ldy are multiples
- * of 4 (FP32 vectors) / 2 (FP64) (tuning override; MAXE_AUTOTUNE times it
- * against the other SpMM paths at k = 16 and keeps the fastest). */
+ * each lane holds a piece of the k columns of X and Y (FP32 vectors: 16 bytes
+ * where X and Y are 16-byte aligned with ldx, ldy multiples of 4, else what their
+ * alignment allows; FP64: one column), a group walks its row's entries and writes
+ * its piece of Y once -- for matrices with short rows (tuning override;
+ * MAXE_AUTOTUNE times it against the other SpMM paths at k = 16 and keeps the
+ * fastest). */
 #define MAXE_SPMM_ROWS 0x400u
 /* Flag of maxe_permute_csr: with MAXE_SPMM_ROWS, each lane group also
  * prefetches into L2 the X rows of its next row while it sums the current one

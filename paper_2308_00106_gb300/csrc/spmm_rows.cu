@@ -18,8 +18,8 @@
 // kChunkE is a chunk of its own; its entries past the staged ones are read
 // from global memory.
 //
-// Entries go eight at a time, their X loads issued together, into four
-// partial sums (entries u and u + 4 of a step share one) added in a fixed
+// Entries go four (16-byte pieces) or eight at a time, their X loads issued
+// together, into four partial sums (entry j of a row: sum j % 4) added in a fixed
 // order at the end: shorter dependency chains and a rounding error that grows
 // with a quarter of the row's length.  The work is cut into parts of about
 // kPartE entries (the handle's nnz-balanced row ranges, each split into Q
@@ -34,9 +34,8 @@
 // aligned column and value arrays and rows of X under 2 GiB.
 //
 // X or Y rows that are not whole 16-byte pieces (an odd k in contiguous
-// tensors) take a variant whose lanes load 16, 8 or 4 (FP64: 16 or 8) bytes,
-// as X's alignment allows, with up to 32 lanes to a row, and store Y column
-// by column: an X row is still read by one load of the group.  Poisson rows of
+// tensors) take a variant whose lanes load 16, 8 or 4 (FP64: 8) bytes, as X's
+// alignment allows, with up to 32 lanes to a row, and store Y column by column: an X row is still read by one load of the group.  Poisson rows of
 // 20, 100,003 rows, FP32, k = 7 contiguous: 58 us in seven column passes, 21 us
 // here (k = 31: 236 -> 42 us; FP64, k = 7: 131 -> 69 us).
 #include "spmm_rows.cuh"
@@ -81,9 +80,17 @@ __device__ __forceinline__ bool next_start(const RowsParams& p, int32_t* r, int6
   return true;
 }
 
-// GC: lanes per row (0: p.G, a power of two); VC, YVEC: see rows_chunk.
+// CTAs per SM the registers are cut for: FP64 sums take twice the registers.
+template <typename AT>
+constexpr int rows_blocks() {
+  return sizeof(AT) == 8 ? 3 : 4;
+}
+
+// GC: lanes per row (0: p.G, a power of two; a constant is worth 10% on rows of
+// 40); VC, YVEC: see rows_chunk.
 template <typename VT, int GC, int VC, bool YVEC>
-__global__ void __launch_bounds__(kRowsThreads) spmm_rows_kernel(const RowsParams p) {
+__global__ void __launch_bounds__(kRowsThreads, rows_blocks<typename RowsT<VT>::AT>())
+    spmm_rows_kernel(const RowsParams p) {
   extern __shared__ __align__(16) unsigned char rows_smem[];
   const int G = GC ? GC : p.G;
   const int lane = threadIdx.x & 31, sub = lane % G, grp = lane / G;
@@ -153,25 +160,35 @@ template <typename VT>
 maxe_status launch_rows(RowsParams p, int sms, cudaStream_t st) {
   using AT = typename RowsT<VT>::AT;
   constexpr int VC = RowsT<VT>::VC;
-  // columns per load that X's rows allow: 16 bytes, 8 (FP32) or one column
+  // columns per load that FP32 rows of X allow: 16 bytes, 8 or one column
   auto whole = [](const void* q, int64_t ld, int vc) {
     return ld % vc == 0 && reinterpret_cast<uintptr_t>(q) % (vc * sizeof(AT)) == 0;
   };
-  if (whole(p.op.X, p.op.ldx, VC) && whole(p.op.Y, p.op.ldy, VC)) {
-    switch (rows_group<VT>(p.op.k)) {
-      case 1: return launch_rows_g<VT, 1>(p, sms, st);
-      case 2: return launch_rows_g<VT, 2>(p, sms, st);
-      case 4: return launch_rows_g<VT, 4>(p, sms, st);
-      default: return launch_rows_g<VT, 8>(p, sms, st);
+  if constexpr (RowsT<VT>::kLaneCols == 1) {  // FP64: see there
+    switch (rows_lanes(p.op.k)) {
+      case 1: return launch_rows_g<VT, 1, 1, false>(p, sms, st);
+      case 2: return launch_rows_g<VT, 2, 1, false>(p, sms, st);
+      case 4: return launch_rows_g<VT, 4, 1, false>(p, sms, st);
+      case 8: return launch_rows_g<VT, 8, 1, false>(p, sms, st);
+      case 16: return launch_rows_g<VT, 16, 1, false>(p, sms, st);
+      default: return launch_rows_g<VT, 32, 1, false>(p, sms, st);
     }
-  }
-  const int vc = whole(p.op.X, p.op.ldx, VC) ? VC : (whole(p.op.X, p.op.ldx, 2) ? 2 : 1);
-  p.G = 1;  // a lane per piece of the row, at most 32 (more pieces: passes)
-  while (p.G < 32 && p.G * vc < p.op.k) p.G *= 2;
-  if (vc == VC) return launch_rows_g<VT, 0, VC, false>(p, sms, st);
-  if constexpr (VC == 4)
+  } else {
+    if (whole(p.op.X, p.op.ldx, VC) && whole(p.op.Y, p.op.ldy, VC)) {
+      switch (rows_lanes((p.op.k + VC - 1) / VC)) {
+        case 1: return launch_rows_g<VT, 1>(p, sms, st);
+        case 2: return launch_rows_g<VT, 2>(p, sms, st);
+        case 4: return launch_rows_g<VT, 4>(p, sms, st);
+        case 8: return launch_rows_g<VT, 8>(p, sms, st);
+        default: return launch_rows_g<VT, 16>(p, sms, st);
+      }
+    }
+    const int vc = whole(p.op.X, p.op.ldx, 4) ? 4 : (whole(p.op.X, p.op.ldx, 2) ? 2 : 1);
+    p.G = rows_lanes((p.op.k + vc - 1) / vc);
+    if (vc == 4) return launch_rows_g<VT, 0, 4, false>(p, sms, st);
     if (vc == 2) return launch_rows_g<VT, 0, 2, false>(p, sms, st);
-  return launch_rows_g<VT, 0, 1, false>(p, sms, st);
+    return launch_rows_g<VT, 0, 1, false>(p, sms, st);
+  }
 }
 
 }  // namespace

@@ -7,12 +7,12 @@
 // into one half of the warp's double buffer (16-byte cp.async copies rounded
 // out to 8-entry boundaries; the CSR arrays are padded past nnz) and writes its
 // row pointers; rows_chunk multiplies the rows of a staged chunk, a group of G
-// lanes per row, each lane a 16-byte piece of the X and Y rows (VC = 4 FP32 or
-// 2 FP64 columns), gathering X pieces by the staged column indices and
-// accumulating in registers.  Entries go eight at a time, their X loads issued
-// together, into four partial sums (entries u and u + 4 of a step share one)
-// added in a fixed order, so a Y row is one group's sum in a fixed order: the
-// same bits whichever warp, launch or batch computes it.  A row longer than
+// lanes per row, each lane a piece of VC columns of the X and Y rows (4 FP32
+// columns where rows are 16-byte aligned), gathering X pieces by the staged
+// column indices and accumulating in registers.  Entries go four or eight at a
+// time, their X loads issued together, into four partial sums (entry j of a row:
+// sum j % 4) added in a fixed order, so a Y row is one group's sum in a fixed
+// order: the same bits whichever warp, launch or batch computes it.  A row longer than
 // kChunkE is a chunk of its own; its entries past the staged ones are read
 // from global memory.
 #pragma once
@@ -22,7 +22,7 @@
 namespace maxe {
 namespace rows {
 
-constexpr int kRowsUnroll = 8;  // entries per step of a group
+constexpr int kRowsAhead = 8;   // entries of the next row prefetched, per lane of the group
 constexpr int kRowsParts = 4;   // partial sums of a group
 constexpr int kChunkE = 256;    // entries of a chunk (a longer row: the first kChunkE)
 constexpr int kChunkR = 63;     // rows of a chunk: its 64 row pointers are two per lane
@@ -33,19 +33,27 @@ struct RowsT;
 template <>
 struct RowsT<float> {
   using AT = float;
-  static constexpr int VC = 4;  // columns of a 16-byte piece
+  static constexpr int VC = 4;         // columns of a 16-byte piece
+  static constexpr int kLaneCols = 4;  // columns a lane takes of aligned rows
   static __device__ __forceinline__ float acc(float v) { return v; }
 };
 template <>
 struct RowsT<uint16_t> {
   using AT = float;
   static constexpr int VC = 4;
+  static constexpr int kLaneCols = 4;
   static __device__ __forceinline__ float acc(uint16_t v) { return __uint_as_float(static_cast<uint32_t>(v) << 16); }
 };
 template <>
 struct RowsT<double> {
   using AT = double;
   static constexpr int VC = 2;
+  // One column a lane whatever the alignment: twice the lanes a row, so half the
+  // rows a warp, which costs fewer bank conflicts of the staged entries and less
+  // waiting for the longest row than 16-byte loads save.  300,000 rows of 40, k = 4:
+  // 352 -> 184 us, k = 16: 604 -> 436 us; permuted 2048 x 2048 Laplacian 534 -> 397
+  // and 1300 -> 1250 us.
+  static constexpr int kLaneCols = 1;
   static __device__ __forceinline__ double acc(double v) { return v; }
 };
 
@@ -216,6 +224,61 @@ __device__ __forceinline__ int32_t stage_chunk(RowsStage<VT>* s, int buf, const 
   return n;
 }
 
+// U entries of a row from t on (PRED: only the first `left` of them), their X
+// loads issued together: entry u goes to partial sum u % kRowsParts.  COL and VAL:
+// the row's column indices and values, in shared or global memory.
+template <typename VT, int VC, int U, bool PRED>
+__device__ __forceinline__ void rows_step(typename RowsPiece<typename RowsT<VT>::AT, VC>::V (&part)[kRowsParts],
+                                          const int32_t* col, const VT* val, int left, const char* xc,
+                                          int32_t ldx_bytes) {
+  using T = RowsT<VT>;
+  using AT = typename T::AT;
+  using V = typename RowsPiece<AT, VC>::V;
+  V xv[U];
+  AT av[U];
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    if (PRED) {
+      av[u] = AT(0);
+      zero(xv[u]);
+    }
+    if (!PRED || u < left) {
+      // X piece of row COL: xc + COL * ldx_bytes (one wide multiply-add per entry)
+      xv[u] = __ldg(reinterpret_cast<const V*>(xc + static_cast<int64_t>(col[u]) * static_cast<int64_t>(ldx_bytes)));
+      av[u] = T::acc(val[u]);
+    }
+  }
+#pragma unroll
+  for (int u = 0; u < U; ++u) fma_vec(part[u % kRowsParts], av[u], xv[u]);
+}
+
+// Entries of a row, n of them: whole steps of U entries without predicates, then
+// one of kRowsParts, then a predicated rest.  Every step starts at a multiple of
+// kRowsParts, so entry j of the row is in partial sum j % kRowsParts whatever U.
+template <typename VT, int VC, int U>
+__device__ __forceinline__ void rows_entries(typename RowsPiece<typename RowsT<VT>::AT, VC>::V (&part)[kRowsParts],
+                                             const int32_t* col, const VT* val, int32_t n, const char* xc,
+                                             int32_t ldx_bytes) {
+  static_assert(U % kRowsParts == 0, "steps keep the entries' partial sums");
+  int32_t t = 0;
+#pragma unroll 1
+  for (; t + U <= n; t += U) rows_step<VT, VC, U, false>(part, col + t, val + t, U, xc, ldx_bytes);
+  if (U > kRowsParts && t + kRowsParts <= n) {
+    rows_step<VT, VC, kRowsParts, false>(part, col + t, val + t, kRowsParts, xc, ldx_bytes);
+    t += kRowsParts;
+  }
+  if (t < n) rows_step<VT, VC, kRowsParts - 1, true>(part, col + t, val + t, n - t, xc, ldx_bytes);
+}
+
+// Entries per whole step: as many as keep their X pieces in registers.  Eight
+// 16-byte pieces do not fit beside the rest in 64 registers: the compiler then
+// loads them one after the other (BF16 values: 175 us against 105 with four, on
+// 300,000 rows of 40, k = 16).
+template <typename AT, int VC>
+constexpr int rows_unroll() {
+  return sizeof(AT) * VC >= 16 ? 4 : 8;
+}
+
 // Multiplies the rows of chunk buffer `buf` and writes their Y pieces: lane
 // `sub` of group `grp` (G lanes per group, GPW = 32 / G groups per warp), each
 // lane VC columns.  YVEC: Y rows are 16-byte aligned and VC is a whole 16 bytes.
@@ -226,91 +289,63 @@ __device__ __forceinline__ void rows_chunk(const RowsStage<VT>* s, int buf, cons
   using T = RowsT<VT>;
   using AT = typename T::AT;
   using V = typename RowsPiece<AT, VC>::V;
+  constexpr int U = rows_unroll<AT, VC>();
   const int32_t ldx_bytes = static_cast<int32_t>(p.ldx * static_cast<int64_t>(sizeof(AT)));  // < 2^31 (checked)
-  const int64_t ldyv = p.ldy / VC;
   const int kv = (p.k + VC - 1) / VC;
   const int32_t* scol = s->col[buf];
   const VT* sval = s->val[buf];
-  const int64_t e0a = s->e0a[buf];
-  const int32_t r0 = s->r[buf], n = s->n[buf], lim = s->lim[buf];
-  const int32_t* gcol = p.col + e0a;
-  const VT* gval = static_cast<const VT*>(p.val) + e0a;
+  const int32_t n = s->n[buf], lim = s->lim[buf];
   for (int j = grp; j < n; j += GPW) {
     const int32_t t0 = s->rp[buf][j], t1 = s->rp[buf][j + 1];
-    const int64_t yr = p.yperm ? static_cast<int64_t>(__ldg(p.yperm + r0 + j)) : static_cast<int64_t>(r0 + j);
     const int32_t ts = min(t1, lim);  // staged entries of the row end here
     // the X rows of the group's next row into L2, one line each (when a row
     // spans several lanes: with one lane per row the prefetches cost more)
     if (p.pf && G > 1 && j + GPW < n) {
       const int32_t u0 = s->rp[buf][j + GPW], u1 = min(s->rp[buf][j + GPW + 1], lim);
-      for (int32_t u = u0 + sub; u < u1 && u < u0 + kRowsUnroll * G; u += G)
+      for (int32_t u = u0 + sub; u < u1 && u < u0 + kRowsAhead * G; u += G)
         asm volatile("prefetch.global.L2 [%0];" ::"l"(static_cast<const char*>(p.X) +
                                                        static_cast<int64_t>(scol[u]) * static_cast<int64_t>(ldx_bytes)));
     }
     for (int c = sub; c < kv; c += G) {
-      // X piece c of row COL: xc + COL * ldx_bytes (one wide multiply-add per entry)
       const char* xc = static_cast<const char*>(p.X) + static_cast<int>(sizeof(V)) * c;
       V part[kRowsParts];
 #pragma unroll
       for (int u = 0; u < kRowsParts; ++u) zero(part[u]);
-      for (int32_t t = t0; t < ts; t += kRowsUnroll) {
-        AT av[kRowsUnroll];
-        V xv[kRowsUnroll];
-#pragma unroll
-        for (int u = 0; u < kRowsUnroll; ++u) {
-          av[u] = AT(0);
-          zero(xv[u]);
-          if (t + u < ts) {
-            av[u] = T::acc(sval[t + u]);
-            xv[u] = __ldg(reinterpret_cast<const V*>(xc + static_cast<int64_t>(scol[t + u]) *
-                                                              static_cast<int64_t>(ldx_bytes)));
-          }
-        }
-#pragma unroll
-        for (int u = 0; u < kRowsUnroll; ++u) fma_vec(part[u % kRowsParts], av[u], xv[u]);
-      }
-      for (int32_t t = max(t0, ts); t < t1; t += kRowsUnroll) {  // past the staged part of a long row
-        AT av[kRowsUnroll];
-        V xv[kRowsUnroll];
-#pragma unroll
-        for (int u = 0; u < kRowsUnroll; ++u) {
-          av[u] = AT(0);
-          zero(xv[u]);
-          if (t + u < t1) {
-            av[u] = T::acc(gval[t + u]);
-            xv[u] = __ldg(reinterpret_cast<const V*>(xc + static_cast<int64_t>(__ldg(gcol + t + u)) *
-                                                              static_cast<int64_t>(ldx_bytes)));
-          }
-        }
-#pragma unroll
-        for (int u = 0; u < kRowsUnroll; ++u) fma_vec(part[u % kRowsParts], av[u], xv[u]);
+      rows_entries<VT, VC, U>(part, scol + t0, sval + t0, ts - t0, xc, ldx_bytes);
+      // Past the staged part of a long row; it ends kChunkE entries into the
+      // row, so the partial sums go on where they were.
+      if (t1 > ts) {
+        const int64_t e = s->e0a[buf] + ts;
+        rows_entries<VT, VC, U>(part, p.col + e, static_cast<const VT*>(p.val) + e, t1 - ts, xc, ldx_bytes);
       }
       add_vec(part[0], part[1]);
       add_vec(part[2], part[3]);
       add_vec(part[0], part[2]);
+      const int32_t row = s->r[buf] + j;
+      const int64_t yr = p.yperm ? static_cast<int64_t>(__ldg(p.yperm + row)) : static_cast<int64_t>(row);
       if constexpr (YVEC)
-        store_piece(static_cast<V*>(p.Y) + yr * ldyv + c, part[0], p.k - c * VC);
+        store_piece(reinterpret_cast<V*>(static_cast<AT*>(p.Y) + yr * p.ldy) + c, part[0], p.k - c * VC);
       else
         store_columns(static_cast<AT*>(p.Y) + yr * p.ldy + c * VC, part[0], p.k - c * VC);
     }
   }
 }
 
-// Lane group of a product with k columns: one lane per 16-byte piece of a
-// row, at most 8 (more pieces: passes over the row).
-template <typename VT>
-__host__ __device__ __forceinline__ int rows_group(int k) {
-  const int kv = (k + RowsT<VT>::VC - 1) / RowsT<VT>::VC;
-  return kv <= 1 ? 1 : (kv <= 2 ? 2 : (kv <= 4 ? 4 : 8));
+// Lanes of a row with `pieces` pieces: a power of two, at most 32 (more pieces: passes).
+__host__ __device__ __forceinline__ int rows_lanes(int pieces) {
+  int g = 1;
+  while (g < 32 && g < pieces) g *= 2;
+  return g;
 }
 
 // Rows [r_lo, b) of the product by one warp: chunk c is multiplied while the
 // indices of chunk c + 1 load into the other buffer and the row pointers of
 // chunk c + 2 into registers.  Warp-uniform; all 32 lanes take part.
-template <typename VT>
-__device__ __forceinline__ void rows_range(RowsStage<VT>* s, const RowsOperand& p, int32_t r_lo, int32_t b, int G,
+template <typename VT, int VC, bool YVEC, int GC>
+__device__ __forceinline__ void rows_range(RowsStage<VT>* s, const RowsOperand& p, int32_t r_lo, int32_t b, int Gr,
                                            int lane) {
   if (r_lo >= b) return;
+  const int G = GC ? GC : Gr;
   const int GPW = 32 / G, sub = lane % G, grp = lane / G;
   int32_t pa, pb;
   load_rp(p.rowptr, r_lo, b, lane, &pa, &pb);
@@ -325,7 +360,7 @@ __device__ __forceinline__ void rows_range(RowsStage<VT>* s, const RowsOperand& 
       r2 = r1 + stage_chunk<VT>(s, buf ^ 1, p, r1, b, lane, pa, pb);
       if (r2 < b) load_rp(p.rowptr, r2, b, lane, &pa, &pb);
     }
-    rows_chunk<VT>(s, buf, p, G, GPW, grp, sub);
+    rows_chunk<VT, VC, YVEC>(s, buf, p, G, GPW, grp, sub);
     __syncwarp();
     if (r1 >= b) break;
     r1 = r2;
