@@ -78,6 +78,15 @@ namespace maxe {
 inline int value_bytes(maxe_dtype d) { return d == MAXE_F64 ? 8 : (d == MAXE_F32 ? 4 : 2); }
 inline int vector_bytes(maxe_dtype d) { return d == MAXE_F64 ? 8 : 4; }
 
+// Whether the arrays of a product with k columns leave no room to find them in L2
+// again (129 MB, of which a quarter is left to others): such a product streams
+// its matrix past x.
+inline bool beyond_l2(const maxe_handle* h, int64_t k) {
+  const int64_t bytes = h->nnz * (4 + value_bytes(h->dtype)) + 4 * static_cast<int64_t>(h->rows) +
+                        (static_cast<int64_t>(h->rows) + h->cols) * k * vector_bytes(h->dtype);
+  return bytes > (int64_t(96) << 20);
+}
+
 // perm.cu: out = first .. first + n - 1 in ascending (key(seed, tag, i), i) order.
 size_t perm_order_scratch_bytes(int64_t n);
 maxe_status perm_order(uint64_t seed, int32_t tag, int32_t first, int32_t n, int32_t* out, void* scratch,

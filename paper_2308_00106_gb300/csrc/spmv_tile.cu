@@ -20,9 +20,9 @@
 //
 // Random gathers are bound by the L1 tag stage, one line a cycle and SM (292
 // G/s; 240 G/s reached while x stays in L2).  Permuted Laplacian, FP32, warp
-// kernel -> tiles: 4096 x 4096 646 -> 416 us (x of 67 MB no longer fits in L2
-// beside the stream), 2048 x 2048 97 -> 91 us; natural order, x in L1: 4096 x
-// 4096 215 -> 175 us, FP64 464 -> 271 us.  With longer rows (Poisson, 15 to 50
+// kernel -> tiles: 4096 x 4096 646 -> 372 us (x of 67 MB no longer fits in L2
+// beside the stream), 2048 x 2048 97 -> 89 us; natural order, x in L1: 4096 x
+// 4096 215 -> 174 us, FP64 464 -> 271 us.  With longer rows (Poisson, 15 to 50
 // a row) the two are even and FP64 loses (150 -> 185 us at 20M entries), so the
 // autotuner times all and takes the tiles where they are 5% faster; a handle that
 // was not tuned keeps the warp kernel.
@@ -69,9 +69,59 @@ struct TileParams {
   int shift;  // log2 of G, lanes per row
 };
 
-__device__ __forceinline__ void tile_cp16(void* dst, const void* src) {
+// Loads of a product that does not fit in L2 (BIG): the matrix, its row pointers
+// and y pass through as the first to go, x is what should stay.  One that fits is
+// read again by the next product and keeps plain loads (4096 x 4096 permuted
+// Laplacian, FP32: 424 us plain, 380 us so; 1000 x 1000: 25 us plain, 27 us so,
+// FP64 44 and 54 us).
+struct TilePolicy {
+  uint64_t once, keep;
+};
+__device__ __forceinline__ TilePolicy tile_policy() {
+  TilePolicy p;
+  asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p.once));
+  asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(p.keep));
+  return p;
+}
+
+template <bool BIG>
+__device__ __forceinline__ void tile_cp16(void* dst, const void* src, const TilePolicy& pol) {
   const uint32_t d = static_cast<uint32_t>(__cvta_generic_to_shared(dst));
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
+  if constexpr (BIG)
+    asm volatile("cp.async.cg.shared.global.L2::cache_hint [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "l"(pol.once)
+                 : "memory");
+  else
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
+}
+template <bool BIG>
+__device__ __forceinline__ int4 tile_cols(const int32_t* p, const TilePolicy& pol) {
+  if constexpr (!BIG) return __ldcs(reinterpret_cast<const int4*>(p));
+  int4 v;
+  asm volatile("ld.global.nc.L1::no_allocate.L2::cache_hint.v4.s32 {%0, %1, %2, %3}, [%4], %5;"
+               : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+               : "l"(p), "l"(pol.once));
+  return v;
+}
+template <bool BIG>
+__device__ __forceinline__ int32_t tile_rowptr(const int32_t* p, const TilePolicy& pol) {
+  if constexpr (!BIG) return __ldg(p);
+  int32_t v;
+  asm volatile("ld.global.nc.L2::cache_hint.s32 %0, [%1], %2;" : "=r"(v) : "l"(p), "l"(pol.once));
+  return v;
+}
+template <bool BIG>
+__device__ __forceinline__ float tile_x(const float* p, const TilePolicy& pol) {
+  if constexpr (!BIG) return *p;
+  float v;
+  asm volatile("ld.global.L2::cache_hint.f32 %0, [%1], %2;" : "=f"(v) : "l"(p), "l"(pol.keep));
+  return v;
+}
+template <bool BIG>
+__device__ __forceinline__ double tile_x(const double* p, const TilePolicy& pol) {
+  if constexpr (!BIG) return *p;
+  double v;
+  asm volatile("ld.global.L2::cache_hint.f64 %0, [%1], %2;" : "=d"(v) : "l"(p), "l"(pol.keep));
+  return v;
 }
 
 template <typename AT>
@@ -84,7 +134,7 @@ __device__ __forceinline__ void sts4(AT* p, const AT (&v)[4]) {
   }
 }
 
-template <typename VT>
+template <typename VT, bool BIG>
 __global__ void __launch_bounds__(kTileThreads, 6) spmv_tile_kernel(const TileParams p) {
   using T = TileT<VT>;
   using AT = typename T::AT;
@@ -102,28 +152,29 @@ __global__ void __launch_bounds__(kTileThreads, 6) spmv_tile_kernel(const TilePa
   // Whole 16-byte pieces: slots past n hold entries of later tiles or the
   // arrays' padding (columns within the matrix), and are not read back.
   const int32_t* col = p.col + base;
+  const TilePolicy pol = BIG ? tile_policy() : TilePolicy{};
   int4 c[kTileItems / 4];
 #pragma unroll
   for (int j = 0; j < kTileItems / 4; ++j) {
     const int s = 4 * (t + j * kTileThreads);
-    if (s < n) c[j] = __ldcs(reinterpret_cast<const int4*>(col + s));
+    if (s < n) c[j] = tile_cols<BIG>(col + s, pol);
   }
   constexpr int per = 16 / static_cast<int>(sizeof(VT));
   const VT* val = static_cast<const VT*>(p.val) + base;
 #pragma unroll
   for (int j = 0; j < kTileItems / per; ++j) {
     const int s = per * (t + j * kTileThreads);
-    if (s < n) tile_cp16(vs + s, val + s);
+    if (s < n) tile_cp16<BIG>(vs + s, val + s, pol);
   }
   asm volatile("cp.async.commit_group;" ::: "memory");
   AT xv[kTileItems / 4][4];
 #pragma unroll
   for (int j = 0; j < kTileItems / 4; ++j) {
     if (4 * (t + j * kTileThreads) < n) {
-      xv[j][0] = x[c[j].x];
-      xv[j][1] = x[c[j].y];
-      xv[j][2] = x[c[j].z];
-      xv[j][3] = x[c[j].w];
+      xv[j][0] = tile_x<BIG>(x + c[j].x, pol);
+      xv[j][1] = tile_x<BIG>(x + c[j].y, pol);
+      xv[j][2] = tile_x<BIG>(x + c[j].z, pol);
+      xv[j][3] = tile_x<BIG>(x + c[j].w, pol);
     }
   }
   // the row pointers of the first rows come in under the gathers
@@ -132,8 +183,8 @@ __global__ void __launch_bounds__(kTileThreads, 6) spmv_tile_kernel(const TilePa
   uint32_t rr = r0 + (t >> shift);
   int32_t s = 0, e = 0;
   if (rr < r1) {
-    s = static_cast<int32_t>(__ldg(p.rowptr + rr) - base);
-    e = static_cast<int32_t>(__ldg(p.rowptr + rr + 1) - base);
+    s = static_cast<int32_t>(tile_rowptr<BIG>(p.rowptr + rr, pol) - base);
+    e = static_cast<int32_t>(tile_rowptr<BIG>(p.rowptr + rr + 1, pol) - base);
   }
 #pragma unroll
   for (int j = 0; j < kTileItems / 4; ++j) {
@@ -180,13 +231,15 @@ __global__ void __launch_bounds__(kTileThreads, 6) spmv_tile_kernel(const TilePa
     if (have && sub == 0) {
       if (e > n)
         part[kTileWarps] = acc;  // the tile's last row runs on past the staged entries
+      else if (BIG && !p.yperm)  // (scattered y is put together in L2)
+        __stcs(y + rr, acc);
       else
         y[p.yperm ? __ldg(p.yperm + rr) : rr] = acc;
     }
     rr += rows;
     if (rr < r1) {
-      s = static_cast<int32_t>(__ldg(p.rowptr + rr) - base);
-      e = static_cast<int32_t>(__ldg(p.rowptr + rr + 1) - base);
+      s = static_cast<int32_t>(tile_rowptr<BIG>(p.rowptr + rr, pol) - base);
+      e = static_cast<int32_t>(tile_rowptr<BIG>(p.rowptr + rr + 1, pol) - base);
     }
   }
   if (all <= kTileCap) return;
@@ -221,6 +274,17 @@ __global__ void tile_starts_kernel(const int32_t* __restrict__ first, const int3
   tile[b] = make_int2(r, rowptr[r]);
 }
 
+template <typename VT>
+maxe_status tile_launch(const TileParams& p, const maxe_handle* h, cudaStream_t st) {
+  const unsigned grid = static_cast<unsigned>(h->tiles);
+  if (beyond_l2(h, 1))
+    spmv_tile_kernel<VT, true><<<grid, kTileThreads, 0, st>>>(p);
+  else
+    spmv_tile_kernel<VT, false><<<grid, kTileThreads, 0, st>>>(p);
+  MAXE_CUDA_TRY(cudaGetLastError());
+  return MAXE_OK;
+}
+
 }  // namespace
 
 maxe_status spmv_tile_build(maxe_handle* h, cudaStream_t st) {
@@ -248,15 +312,12 @@ maxe_status spmv_tile_build(maxe_handle* h, cudaStream_t st) {
 
 maxe_status spmv_tile_launch(const maxe_handle* h, const void* x, void* y, const int32_t* yperm, cudaStream_t st) {
   TileParams p{h->rowptr, h->col, h->val, h->tile, x, y, yperm, h->tile_shift};
-  const unsigned grid = static_cast<unsigned>(h->tiles);
   switch (h->dtype) {
-    case MAXE_F64: spmv_tile_kernel<double><<<grid, kTileThreads, 0, st>>>(p); break;
-    case MAXE_F32: spmv_tile_kernel<float><<<grid, kTileThreads, 0, st>>>(p); break;
-    case MAXE_BF16: spmv_tile_kernel<uint16_t><<<grid, kTileThreads, 0, st>>>(p); break;
-    default: return MAXE_ERR_INVALID;
+    case MAXE_F64: return tile_launch<double>(p, h, st);
+    case MAXE_F32: return tile_launch<float>(p, h, st);
+    case MAXE_BF16: return tile_launch<uint16_t>(p, h, st);
   }
-  MAXE_CUDA_TRY(cudaGetLastError());
-  return MAXE_OK;
+  return MAXE_ERR_INVALID;
 }
 
 }  // namespace maxe
