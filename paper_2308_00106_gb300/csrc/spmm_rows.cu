@@ -53,6 +53,7 @@ struct RowsParams {
   RowsOperand op;
   const int32_t* wrow;
   int32_t nW, Q;
+  bool once;   // see the kernel's ONCE
   int32_t G;   // lanes per row, where the kernel has none of its own
   int64_t NG;  // warps of the grid: warp g takes parts g, g + NG, g + 2 NG, ...
 };
@@ -88,7 +89,11 @@ constexpr int rows_blocks() {
 
 // GC: lanes per row (0: p.G, a power of two; a constant is worth 10% on rows of
 // 40); VC, YVEC: see rows_chunk.
-template <typename VT, int GC, int VC, bool YVEC>
+// ONCE: the matrix leaves L2 first, so that X stays: where X rows are gathered at
+// random and the product does not fit in L2 (permuted 2048 x 2048 Laplacian, k = 4:
+// FP32 153 -> 137 us, BF16 124 -> 114 us).  A stencil's X rows are there anyway, and
+// its product is 2% slower so.
+template <typename VT, int GC, int VC, bool YVEC, bool ONCE>
 __global__ void __launch_bounds__(kRowsThreads, rows_blocks<typename RowsT<VT>::AT>())
     spmm_rows_kernel(const RowsParams p) {
   extern __shared__ __align__(16) unsigned char rows_smem[];
@@ -107,7 +112,7 @@ __global__ void __launch_bounds__(kRowsThreads, rows_blocks<typename RowsT<VT>::
   int32_t pa, pb;
   load_rp(p.op.rowptr, r1, b1, lane, &pa, &pb);
   int buf = 0;
-  r1 += stage_chunk<VT>(s, buf, p.op, r1, b1, lane, pa, pb);
+  r1 += stage_chunk<VT, ONCE>(s, buf, p.op, r1, b1, lane, pa, pb);
   bool more = next_start(p, &r1, &P1, &b1);  // (r1, b1): the next chunk
   if (more) load_rp(p.op.rowptr, r1, b1, lane, &pa, &pb);
   while (true) {
@@ -117,7 +122,7 @@ __global__ void __launch_bounds__(kRowsThreads, rows_blocks<typename RowsT<VT>::
     int64_t P2 = P1;
     bool more2 = false;
     if (more) {  // stage the next chunk and fetch the row pointers of the one after
-      r2 += stage_chunk<VT>(s, buf ^ 1, p.op, r1, b1, lane, pa, pb);
+      r2 += stage_chunk<VT, ONCE>(s, buf ^ 1, p.op, r1, b1, lane, pa, pb);
       more2 = next_start(p, &r2, &P2, &b2);
       if (more2) load_rp(p.op.rowptr, r2, b2, lane, &pa, &pb);
     }
@@ -132,18 +137,20 @@ __global__ void __launch_bounds__(kRowsThreads, rows_blocks<typename RowsT<VT>::
   }
 }
 
-template <typename VT, int G, int VC = RowsT<VT>::VC, bool YVEC = true>
+template <typename VT, int G, int VC = RowsT<VT>::VC, bool YVEC = true, bool ONCE = false>
 maxe_status launch_rows_g(RowsParams p, int sms, cudaStream_t st) {
+  if constexpr (!ONCE && (YVEC || sizeof(VT) == 8))
+    if (p.once) return launch_rows_g<VT, G, VC, YVEC, true>(p, sms, st);
   static PerDeviceOnce once;
   static int blocks_per_sm[64];
   constexpr size_t smem = sizeof(RowsStage<VT>) * kRowsWarps;
   int dev = 0;
   MAXE_CUDA_TRY(cudaGetDevice(&dev));
   MAXE_TRY(once.run([dev] {
-    MAXE_CUDA_TRY(cudaFuncSetAttribute(spmm_rows_kernel<VT, G, VC, YVEC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    MAXE_CUDA_TRY(cudaFuncSetAttribute(spmm_rows_kernel<VT, G, VC, YVEC, ONCE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        static_cast<int>(smem)));
     int b = 0;
-    MAXE_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, spmm_rows_kernel<VT, G, VC, YVEC>, kRowsThreads, smem));
+    MAXE_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, spmm_rows_kernel<VT, G, VC, YVEC, ONCE>, kRowsThreads, smem));
     blocks_per_sm[dev] = std::max(b, 1);
     return MAXE_OK;
   }));
@@ -151,7 +158,7 @@ maxe_status launch_rows_g(RowsParams p, int sms, cudaStream_t st) {
   const int64_t parts = static_cast<int64_t>(p.nW) * p.Q;
   p.NG = std::max<int64_t>(1, std::min<int64_t>(parts, static_cast<int64_t>(sms) * blocks_per_sm[dev] * kRowsWarps));
   const unsigned grid = static_cast<unsigned>(ceil_div(p.NG, kRowsWarps));
-  spmm_rows_kernel<VT, G, VC, YVEC><<<grid, kRowsThreads, smem, st>>>(p);
+  spmm_rows_kernel<VT, G, VC, YVEC, ONCE><<<grid, kRowsThreads, smem, st>>>(p);
   MAXE_CUDA_TRY(cudaGetLastError());
   return MAXE_OK;
 }
@@ -219,6 +226,7 @@ maxe_status spmm_rows_launch(const maxe_handle* h, int32_t k, const void* X, int
   p.op.ldy = ldy;
   p.op.k = k;
   p.op.pf = h->spmm_rows_pf;
+  p.once = !h->spmm_rows_pf && beyond_l2(h, k);
   p.wrow = h->wrow[0];
   p.nW = h->nW[0];
   // parts of about kPartE entries: a warp's range cut into Q parts of equal row counts

@@ -145,9 +145,18 @@ __device__ __forceinline__ void zero(double& v) { v = 0.0; }
 __device__ __forceinline__ void zero(float4& v) { v = make_float4(0.f, 0.f, 0.f, 0.f); }
 __device__ __forceinline__ void zero(double2& v) { v = make_double2(0.0, 0.0); }
 
+// ONCE: the bytes are the first to leave L2.
+template <bool ONCE>
 __device__ __forceinline__ void cp_async16(void* dst, const void* src) {
   const uint32_t d = static_cast<uint32_t>(__cvta_generic_to_shared(dst));
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
+  if constexpr (ONCE) {
+    uint64_t pol;
+    asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol));
+    asm volatile("cp.async.cg.shared.global.L2::cache_hint [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "l"(pol)
+                 : "memory");
+  } else {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
+  }
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
@@ -192,7 +201,7 @@ __device__ __forceinline__ void load_rp(const int32_t* rowptr, int32_t r, int32_
 // its column indices and values into buffer `buf` (cp.async, committed) and
 // writes its row pointers and extent; returns its row count.  Warp-uniform; all
 // 32 lanes take part.
-template <typename VT>
+template <typename VT, bool ONCE = false>
 __device__ __forceinline__ int32_t stage_chunk(RowsStage<VT>* s, int buf, const RowsOperand& p, int32_t r, int32_t b,
                                                int lane, int32_t pa, int32_t pb) {
   const int32_t rows = min(kChunkR, b - r);
@@ -207,10 +216,10 @@ __device__ __forceinline__ int32_t stage_chunk(RowsStage<VT>* s, int buf, const 
   const int32_t lim = static_cast<int32_t>(std::min<int64_t>(E1, static_cast<int64_t>(E0) + kChunkE) - e0a);
   const int32_t slots = (lim + 7) & ~7;  // <= kSlotE
   const int32_t* gcol = p.col + e0a;
-  for (int i = lane; i < slots / 4; i += 32) cp_async16(&s->col[buf][4 * i], gcol + 4 * i);
+  for (int i = lane; i < slots / 4; i += 32) cp_async16<ONCE>(&s->col[buf][4 * i], gcol + 4 * i);
   constexpr int per = 16 / static_cast<int>(sizeof(VT));
   const VT* gval = static_cast<const VT*>(p.val) + e0a;
-  for (int i = lane; i < slots / per; i += 32) cp_async16(&s->val[buf][per * i], gval + per * i);
+  for (int i = lane; i < slots / per; i += 32) cp_async16<ONCE>(&s->val[buf][per * i], gval + per * i);
   cp_async_commit();
   const int32_t base = static_cast<int32_t>(static_cast<int64_t>(E0) - e0a);
   if (lane <= n) s->rp[buf][lane] = pa - E0 + base;
