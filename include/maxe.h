@@ -105,7 +105,8 @@ typedef enum { MAXE_F64 = 0, MAXE_F32 = 1, MAXE_BF16 = 2 } maxe_dtype;
 /* Tuning overrides of the x-sliced form (with MAXE_XSLICE or MAXE_AUTOTUNE):
  * MAXE_XS_PAIRS runs every tile on a cluster of two CTAs, one per half of the
  * columns, even when the halves are uneven (FP32 and BF16 values; FP64 values
- * never use pairs); MAXE_XS_SINGLE never does.  Not both. */
+ * use pairs only where the library chooses them: even halves and one wave of
+ * tiles, without either flag); MAXE_XS_SINGLE never does.  Not both. */
 #define MAXE_XS_PAIRS 0x100u
 #define MAXE_XS_SINGLE 0x200u
 /* Flag of maxe_permute_csr: SpMM (k > 1) with one row per group of lanes --

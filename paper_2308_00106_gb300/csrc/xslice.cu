@@ -91,6 +91,15 @@ struct XsCfg<double, 1> {
   static constexpr int kBuffers = 2;
   static constexpr int kSteps = 6;
 };
+// Halves: a tile's accumulators take twice the room, so the slices are narrower,
+// and still a cell holds half as many entries again (4.1 steps against 2.7 on
+// the 2^20-row power-law matrix: 156 -> 126 us with the gather of x before it).
+template <>
+struct XsCfg<double, 2> {
+  static constexpr int kSliceCols = 6144;  // 48 KB
+  static constexpr int kBuffers = 2;
+  static constexpr int kSteps = 6;
+};
 
 template <typename VT, int J>
 constexpr size_t xs_ring_bytes() {
@@ -159,6 +168,11 @@ __device__ __forceinline__ uint32_t map_to_rank(const void* p, uint32_t rank) {
 __device__ __forceinline__ float ld_cluster(uint32_t a, float) {
   float v;
   asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
+  return v;
+}
+__device__ __forceinline__ double ld_cluster(uint32_t a, double) {
+  double v;
+  asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(a) : "memory");
   return v;
 }
 
@@ -1132,9 +1146,9 @@ maxe_status xs_launch(const maxe_handle* h, const void* x, void* y, const int32_
 }
 
 // Clusters of two CTAs of the pair kernel that the device runs at once.
-template <typename ValT>
+template <typename VT, typename ValT>
 int pair_clusters(int device, int sms, size_t smem) {
-  if (xs_prepare<float, ValT, 2>(device) != MAXE_OK) return sms / 2;
+  if (xs_prepare<VT, ValT, 2>(device) != MAXE_OK) return sms / 2;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(2 * static_cast<unsigned>(sms));
   cfg.blockDim = dim3(kXsThreads);
@@ -1147,7 +1161,7 @@ int pair_clusters(int device, int sms, size_t smem) {
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   int n = 0;
-  if (cudaOccupancyMaxActiveClusters(&n, spmv_xslice_kernel<float, ValT, 2, false>, &cfg) != cudaSuccess || n < 1) {
+  if (cudaOccupancyMaxActiveClusters(&n, spmv_xslice_kernel<VT, ValT, 2, false>, &cfg) != cudaSuccess || n < 1) {
     cudaGetLastError();
     return sms / 2;
   }
@@ -1257,10 +1271,21 @@ maxe_status build(maxe_handle* h, cudaStream_t st, bool force, bool force_pair, 
   // ---- tiles: nnz-balanced over the CTAs (pairs) the device runs at once,
   // cut shorter where the rows and virtual rows would not fit in shared memory
   int T_target = h->sms;
-  if (J == 2)
-    T_target = h->dtype == MAXE_BF16 ? pair_clusters<uint16_t>(h->device, h->sms, xs_smem_bytes<VT, J>(cap))
-                                     : pair_clusters<float>(h->device, h->sms, xs_smem_bytes<VT, J>(cap));
+  if constexpr (J == 2) {
+    const size_t smem = xs_smem_bytes<VT, J>(cap);
+    if constexpr (sizeof(VT) == 8)
+      T_target = pair_clusters<double, double>(h->device, h->sms, smem);
+    else
+      T_target = h->dtype == MAXE_BF16 ? pair_clusters<float, uint16_t>(h->device, h->sms, smem)
+                                       : pair_clusters<float, float>(h->device, h->sms, smem);
+  }
   T_target = std::max(T_target, 1);
+  // FP64 accumulators: one wave of pairs, or single CTAs
+  auto waves = [&](int64_t tiles) { return sizeof(VT) == 8 && J == 2 && tiles > T_target; };
+  if (waves(ceil_div(M, cap))) {
+    *built = -1;
+    return MAXE_OK;
+  }
   std::vector<int32_t> trow{0};
   std::vector<HalfPlan> plans;
   std::vector<int64_t> pre;
@@ -1292,6 +1317,10 @@ maxe_status build(maxe_handle* h, cudaStream_t st, bool force, bool force_pair, 
   }
   const int32_t T = static_cast<int32_t>(trow.size()) - 1;
   const int32_t Q = T * J;
+  if (waves(T)) {
+    *built = -1;
+    return MAXE_OK;
+  }
   if (J == 2 && !force_pair) {  // both halves of every tile within 10% of their mean
     for (int32_t t = 0; t < T; ++t) {
       const int64_t a = plans[2 * t].entries, b = plans[2 * t + 1].entries;
@@ -1459,7 +1488,8 @@ maxe_status xslice_build(maxe_handle* h, cudaStream_t st, bool force, int pairs)
   int built = 0;
   maxe_status s = MAXE_OK;
   if (h->dtype == MAXE_F64) {
-    s = build<double, 1>(h, st, force, false, &built);
+    if (pairs == 0) s = build<double, 2>(h, st, force, false, &built);
+    if (s == MAXE_OK && built <= 0) s = build<double, 1>(h, st, force, false, &built);
   } else {
     if (pairs >= 0) s = build<float, 2>(h, st, force, pairs > 0, &built);
     if (s == MAXE_OK && built <= 0 && pairs <= 0) s = build<float, 1>(h, st, force, false, &built);
@@ -1473,7 +1503,9 @@ bool xslice_ready(const maxe_handle* h, const void* x) {
 }
 
 maxe_status xslice_launch(const maxe_handle* h, const void* x, void* y, const int32_t* yperm, cudaStream_t st) {
-  if (h->dtype == MAXE_F64) return xs_launch<double, double, 1>(h, x, y, yperm, st);
+  if (h->dtype == MAXE_F64)
+    return h->xs_pair == 2 ? xs_launch<double, double, 2>(h, x, y, yperm, st)
+                           : xs_launch<double, double, 1>(h, x, y, yperm, st);
   if (h->xs_pair == 2) {
     if (h->dtype == MAXE_F32) return xs_launch<float, float, 2>(h, x, y, yperm, st);
     return xs_launch<float, uint16_t, 2>(h, x, y, yperm, st);
