@@ -15,6 +15,7 @@
 #include <algorithm>
 
 #include "handle.cuh"
+#include "launch.cuh"
 
 namespace maxe {
 namespace {
@@ -358,6 +359,8 @@ template <typename T, typename V>
 __global__ void __launch_bounds__(kGatherThreads) gather_kernel(const int32_t* __restrict__ perm, int64_t n,
                                                                 int row_elems, int shift, const T* __restrict__ in,
                                                                 int64_t ld_in, T* __restrict__ out, int64_t ld_out) {
+  start_next();
+  after_previous();
   constexpr int VE = sizeof(V) / sizeof(T);
   const int rows = kGatherThreads >> shift;  // per step of the block
   const int c0 = (threadIdx.x & ((1 << shift) - 1)) * VE;
@@ -392,8 +395,8 @@ void gather_launch(const int32_t* perm, int64_t n, int64_t row_elems, const void
   int shift = 0;  // lanes per row: a power of two, at most 32
   while (shift < 5 && (static_cast<int64_t>(VE) << shift) < row_elems) ++shift;
   const int64_t rows = static_cast<int64_t>(kGatherThreads >> shift) * kGatherRows;
-  gather_kernel<T, V><<<static_cast<unsigned>(ceil_div(n, rows)), kGatherThreads, 0, st>>>(
-      perm, n, static_cast<int>(row_elems), shift, static_cast<const T*>(in), ld_in, static_cast<T*>(out), ld_out);
+  launch_after(gather_kernel<T, V>, static_cast<unsigned>(ceil_div(n, rows)), kGatherThreads, 0, st, perm, n,
+               static_cast<int>(row_elems), shift, static_cast<const T*>(in), ld_in, static_cast<T*>(out), ld_out);
 }
 
 // 16-byte pieces when rows of more than one element start on 16-byte boundaries on both sides.

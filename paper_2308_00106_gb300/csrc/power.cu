@@ -13,6 +13,7 @@
 #include <algorithm>
 
 #include "handle.cuh"
+#include "launch.cuh"
 
 namespace maxe {
 namespace {
@@ -52,6 +53,8 @@ __global__ void __launch_bounds__(kDotThreads) dot_partial(const T* __restrict__
                                                            const int32_t* __restrict__ Qb, int64_t n,
                                                            double* __restrict__ part_aa,
                                                            double* __restrict__ part_ab) {
+  start_next();
+  after_previous();
   __shared__ double ws[kDotThreads / 32];
   const int64_t per = (n + gridDim.x - 1) / gridDim.x;
   const int64_t lo = blockIdx.x * per, hi = std::min<int64_t>(n, lo + per);
@@ -84,6 +87,8 @@ __global__ void __launch_bounds__(kDotThreads) dot_partial(const T* __restrict__
 // took 21 us (512 dependent FP64 adds behind loads).
 __global__ void __launch_bounds__(kDotThreads) dot_final(const double* __restrict__ part, int nparts,
                                                          double* __restrict__ out) {
+  start_next();
+  after_previous();
   __shared__ double ws[kDotThreads / 32];
   const double t = sum_parts(part, nparts, ws);
   if (threadIdx.x == 0) *out = t;
@@ -103,6 +108,8 @@ __global__ void __launch_bounds__(kDotThreads) scale_gather(const int32_t* __res
                                                             const double* __restrict__ part_vw, int np, int64_t n,
                                                             T* __restrict__ out, T* __restrict__ v,
                                                             double* __restrict__ nrm2, double* __restrict__ vw) {
+  start_next();
+  after_previous();
   __shared__ double ws[kDotThreads / 32];
   __shared__ double inv_s;
   const int64_t i0 = static_cast<int64_t>(blockIdx.x) * (kDotThreads * kScaleItems) + threadIdx.x;
@@ -169,17 +176,16 @@ maxe_status run(const maxe_handle* h, const T* v0, int32_t steps, T* v, double* 
   for (int32_t s = 0; s < steps; ++s) {
     MAXE_TRY(spmm_launch(h, 1, x, 1, w, 1, h->rperm, st, kProduct));
     const bool quotient = hist && s > 0;  // v = the iterate after step s
-    dot_partial<T><<<nb, kDotThreads, 0, st>>>(w, v, nullptr, n, part, quotient ? part_vw : nullptr);
+    MAXE_CUDA_TRY(launch_after(dot_partial<T>, nb, kDotThreads, 0, st, w, v, nullptr, n, part,
+                               quotient ? part_vw : nullptr));
     const bool need_v = !xp || hist || s + 1 == steps;  // v besides the gathered x'
-    scale_gather<T><<<scale_blocks(n), kDotThreads, 0, st>>>(h->cperm, w, part, part_vw, nb, n, xp,
-                                                             need_v ? v : nullptr, nullptr,
-                                                             quotient ? hist + s - 1 : nullptr);
+    MAXE_CUDA_TRY(launch_after(scale_gather<T>, scale_blocks(n), kDotThreads, 0, st, h->cperm, w, part, part_vw, nb, n,
+                               xp, need_v ? v : nullptr, nullptr, quotient ? hist + s - 1 : nullptr));
     MAXE_CUDA_TRY(cudaGetLastError());
   }
   MAXE_TRY(spmm_launch(h, 1, x, 1, w, 1, h->rperm, st, kProduct));
-  dot_partial<T><<<nb, kDotThreads, 0, st>>>(v, w, nullptr, n, nullptr, part_vw);
-  dot_final<<<1, kDotThreads, 0, st>>>(part_vw, nb, lam);
-  MAXE_CUDA_TRY(cudaGetLastError());
+  MAXE_CUDA_TRY(launch_after(dot_partial<T>, nb, kDotThreads, 0, st, v, w, nullptr, n, nullptr, part_vw));
+  MAXE_CUDA_TRY(launch_after(dot_final, 1, kDotThreads, 0, st, part_vw, nb, lam));
   MAXE_CUDA_TRY(cudaMemcpyAsync(lambda_host, lam, sizeof(double), cudaMemcpyDeviceToHost, st));
   if (hist && steps > 0) {
     if (steps > 1)
@@ -193,9 +199,9 @@ maxe_status run(const maxe_handle* h, const T* v0, int32_t steps, T* v, double* 
 template <typename T>
 maxe_status norm_gather(const int32_t* Q, int64_t n, const T* w, T* u, double* scratch, cudaStream_t st) {
   const int nb = dot_blocks(n);
-  dot_partial<T><<<nb, kDotThreads, 0, st>>>(w, nullptr, nullptr, n, scratch, nullptr);
-  scale_gather<T><<<scale_blocks(n), kDotThreads, 0, st>>>(Q, w, scratch, nullptr, nb, n, u, nullptr,
-                                                           scratch + kDotBlocks, nullptr);
+  MAXE_CUDA_TRY(launch_after(dot_partial<T>, nb, kDotThreads, 0, st, w, nullptr, nullptr, n, scratch, nullptr));
+  MAXE_CUDA_TRY(launch_after(scale_gather<T>, scale_blocks(n), kDotThreads, 0, st, Q, w, scratch, nullptr, nb, n, u,
+                             nullptr, scratch + kDotBlocks, nullptr));
   MAXE_CUDA_TRY(cudaGetLastError());
   return MAXE_OK;
 }
@@ -204,9 +210,8 @@ template <typename T>
 maxe_status dot_gather(const int32_t* Q, int64_t n, const T* u, const T* w, double* scratch, double* out,
                        cudaStream_t st) {
   const int nb = dot_blocks(n);
-  dot_partial<T><<<nb, kDotThreads, 0, st>>>(u, w, Q, n, nullptr, scratch);
-  dot_final<<<1, kDotThreads, 0, st>>>(scratch, nb, out);
-  MAXE_CUDA_TRY(cudaGetLastError());
+  MAXE_CUDA_TRY(launch_after(dot_partial<T>, nb, kDotThreads, 0, st, u, w, Q, n, nullptr, scratch));
+  MAXE_CUDA_TRY(launch_after(dot_final, 1, kDotThreads, 0, st, scratch, nb, out));
   return MAXE_OK;
 }
 

@@ -38,6 +38,7 @@
 // alignment allows, with up to 32 lanes to a row, and store Y column by column: an X row is still read by one load of the group.  Poisson rows of
 // 20, 100,003 rows, FP32, k = 7 contiguous: 58 us in seven column passes, 21 us
 // here (k = 31: 236 -> 42 us; FP64, k = 7: 131 -> 69 us).
+#include "launch.cuh"
 #include "spmm_rows.cuh"
 
 namespace maxe {
@@ -97,6 +98,7 @@ template <typename VT, int GC, int VC, bool YVEC, bool ONCE>
 __global__ void __launch_bounds__(kRowsThreads, rows_blocks<typename RowsT<VT>::AT>())
     spmm_rows_kernel(const RowsParams p) {
   extern __shared__ __align__(16) unsigned char rows_smem[];
+  after_previous();
   const int G = GC ? GC : p.G;
   const int lane = threadIdx.x & 31, sub = lane % G, grp = lane / G;
   RowsStage<VT>* s = reinterpret_cast<RowsStage<VT>*>(rows_smem) + (threadIdx.x >> 5);
@@ -158,8 +160,7 @@ maxe_status launch_rows_g(RowsParams p, int sms, cudaStream_t st) {
   const int64_t parts = static_cast<int64_t>(p.nW) * p.Q;
   p.NG = std::max<int64_t>(1, std::min<int64_t>(parts, static_cast<int64_t>(sms) * blocks_per_sm[dev] * kRowsWarps));
   const unsigned grid = static_cast<unsigned>(ceil_div(p.NG, kRowsWarps));
-  spmm_rows_kernel<VT, G, VC, YVEC, ONCE><<<grid, kRowsThreads, smem, st>>>(p);
-  MAXE_CUDA_TRY(cudaGetLastError());
+  MAXE_CUDA_TRY(launch_after(spmm_rows_kernel<VT, G, VC, YVEC, ONCE>, grid, kRowsThreads, smem, st, p));
   return MAXE_OK;
 }
 

@@ -51,8 +51,7 @@ template <typename VT, int VW, int IT, bool UNIT>
 maxe_status launch_variant(const Params& p, cudaStream_t st) {
   MAXE_TRY((prepare_variant<VT, VW, IT, UNIT>()));
   const unsigned grid = static_cast<unsigned>(ceil_div(p.nW, kWarps));
-  spmm_warp_kernel<Cfg<VT, VW, IT, UNIT>><<<grid, kThreads, block_smem<VT, VW, IT>(), st>>>(p);
-  MAXE_CUDA_TRY(cudaGetLastError());
+  MAXE_CUDA_TRY(launch_after(spmm_warp_kernel<Cfg<VT, VW, IT, UNIT>>, grid, kThreads, block_smem<VT, VW, IT>(), st, p));
   return MAXE_OK;
 }
 

@@ -29,6 +29,7 @@
 #include <algorithm>
 
 #include "handle.cuh"
+#include "launch.cuh"
 
 namespace maxe {
 namespace {
@@ -141,6 +142,7 @@ __global__ void __launch_bounds__(kTileThreads, 6) spmv_tile_kernel(const TilePa
   __shared__ __align__(16) AT xs[kTileCap];
   __shared__ __align__(16) VT vs[kTileCap];
   __shared__ AT part[kTileWarps + 1];
+  after_previous();
   const int t = threadIdx.x, lane = t & 31;
   const int2 lo = __ldg(p.tile + blockIdx.x), hi = __ldg(p.tile + blockIdx.x + 1);
   const uint32_t r0 = lo.x, r1 = hi.x;  // unsigned: a step past the last row cannot wrap

@@ -7,6 +7,7 @@
 #include <climits>
 
 #include "handle.cuh"
+#include "launch.cuh"
 
 namespace maxe {
 namespace warp {
@@ -742,6 +743,7 @@ __global__ void __launch_bounds__(kThreads, C::kMinBlocks) spmm_warp_kernel(Para
   if (w >= p.nW) return;
   unsigned char* wsmem = smem_raw + sizeof(WarpSmem<typename C::VT, C::VW, C::IT>) * wib;
   init_ring<C>(wsmem);
+  after_previous();
   uint32_t gi = 0;
   process_range<C>(p, w, wsmem, gi);
 }

@@ -54,6 +54,7 @@
 #include <vector>
 
 #include "handle.cuh"
+#include "launch.cuh"
 
 namespace maxe {
 namespace {
@@ -510,6 +511,7 @@ __global__ void __launch_bounds__(kXsThreads, 1) spmv_xslice_kernel(const XsPara
   const int i0 = p.tl_off[q], i1 = p.tl_off[q + 1];
 
   if (warp == kXsWarps) {  // ---------------------------------------- producer
+    after_previous();  // x may come from the kernel before this one
     if (lane == 0) {
       const uint64_t pol = policy_evict_last();
       uint32_t v = 0;
@@ -571,6 +573,9 @@ __global__ void __launch_bounds__(kXsThreads, 1) spmv_xslice_kernel(const XsPara
         qp = xs_next<G>(p, g, qp, i1, lane, winp);
       }
     }
+    // The form's own arrays (complete since the build) were read under the
+    // previous kernel's tail; y may still be read by it.
+    after_previous();
     int i = i0;          // next slice to wait for
     int slot = 0;        // its ring slot
     uint32_t par = 0;    // and the phase parity of that slot's barrier
@@ -1119,24 +1124,23 @@ maxe_status xs_launch(const maxe_handle* h, const void* x, void* y, const int32_
   const unsigned grid = static_cast<unsigned>(h->xs_ntiles) * J;
   const size_t smem = static_cast<size_t>(h->xs_smem);
   if constexpr (J == 1) {
-    if (h->xs_prefetch)
-      spmv_xslice_kernel<VT, ValT, 1, true><<<grid, kXsThreads, smem, st>>>(p);
-    else
-      spmv_xslice_kernel<VT, ValT, 1, false><<<grid, kXsThreads, smem, st>>>(p);
-    MAXE_CUDA_TRY(cudaGetLastError());
+    MAXE_CUDA_TRY(h->xs_prefetch ? launch_after(spmv_xslice_kernel<VT, ValT, 1, true>, grid, kXsThreads, smem, st, p)
+                                 : launch_after(spmv_xslice_kernel<VT, ValT, 1, false>, grid, kXsThreads, smem, st, p));
   } else {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(kXsThreads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = 2;
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // as launch_after
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = 2;
     if (h->xs_prefetch)
       MAXE_CUDA_TRY(cudaLaunchKernelEx(&cfg, spmv_xslice_kernel<VT, ValT, 2, true>, p));
     else
