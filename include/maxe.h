@@ -287,7 +287,8 @@ MAXE_API maxe_status maxe_nnz_entropy_noalloc(const maxe_handle* h, int32_t gr, 
  * product's epilogue, so y = A x.  With MAXE_VEC_PERMUTED, y = A' x directly.
  * x: (device) cols elements, y: (device) rows elements; FP64 for MAXE_F64
  * handles, FP32 otherwise.  x and y must not overlap.  Calls on one handle
- * without MAXE_VEC_PERMUTED share its x' scratch: do not overlap them in time. */
+ * without MAXE_VEC_PERMUTED share its x' scratch (and the y' scratch of large
+ * autotuned handles): do not overlap them in time. */
 MAXE_API maxe_status maxe_spmv(const maxe_handle* h, const void* x, void* y, uint32_t flags, void* stream);
 
 /* a6 + a5 by the staged-tile kernel, whichever kernel maxe_spmv takes for this

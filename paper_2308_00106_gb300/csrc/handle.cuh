@@ -7,6 +7,7 @@
 //   wrow    [nW + 1]                       SpMV work partition: first row of each warp range
 //   rperm, cperm [rows], [cols]            copies of the permutations (or NULL)
 //   xbuf                                   x' = P_c^{-1} x scratch for original-space calls
+//   rinv [rows], ybuf                      large matrices (MAXE_AUTOTUNE): P_r as a gather, and its y' scratch
 //   coo_row [nnz], coo_carry               COO form (MAXE_COO): row of each entry, and
 //                                          per-256-entry-chunk partial sums + flags
 // nnz_pad leaves at least two 128-entry pieces of zeros after the last entry,
@@ -67,6 +68,9 @@ struct maxe_handle {
   void* coo_carry = nullptr;               // COO per-chunk partial sums and flags
   void* xbuf = nullptr;  // cols * k_cap vector elements
   int32_t xbuf_k = 0;
+  int32_t* rinv = nullptr;  // inverse of rperm, where Y rows may be put in order by a second pass
+  void* ybuf = nullptr;     // its y' scratch (original-space calls): rows * ybuf_k vector elements
+  int32_t ybuf_k = 0;
   maxe::Allocator al;
   int device = 0;
   int sms = 0;

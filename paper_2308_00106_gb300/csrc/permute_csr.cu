@@ -58,9 +58,9 @@ struct SortSmem {
 // bin is the number of smaller (column, position) pairs in it, of which there
 // are few.  Any columns are ordered right; uneven ones only make the bins
 // fuller (n^2 / 512 comparisons per thread at the worst).  A bitonic sort of
-// 64-bit keys took 1874 us for 25.4 M entries (2^20 rows), this took 428 us with two
-// CTAs an SM and takes 390 us with three (40 registers, a few spilled): ten barriers
-// a bucket leave a CTA waiting more than it works.
+// 64-bit keys took 1874 us for 25.4 M entries (2^20 rows), this took 417 us with two
+// CTAs an SM and takes 406 us with three (40 registers, a few spilled), with ten
+// barriers a bucket that leave a CTA waiting.
 template <typename VT>
 __global__ void __launch_bounds__(kSortThreads, 3) bucket_sort_kernel(
     const int32_t* __restrict__ rowptr, const int32_t* __restrict__ col, const VT* __restrict__ val,
