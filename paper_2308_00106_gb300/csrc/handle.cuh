@@ -36,6 +36,7 @@ struct maxe_handle {
   int2* tile = nullptr;                    // staged-tile SpMV (MAXE_AUTOTUNE): [tiles + 1] first row, its first entry
   int64_t tiles = 0;
   int tile_shift = 0;                      // log2 of its lanes per row
+  int tile_dense = 0;                      // its variant of more CTAs per SM (autotuned)
   int tile_use = 0;                        // SpMV (k = 1) takes the staged-tile kernel (autotuned)
   int32_t* bwrow = nullptr;                // batch plan: partition with bH entries per warp task
   int32_t bnW = 0;

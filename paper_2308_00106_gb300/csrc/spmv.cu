@@ -264,9 +264,12 @@ maxe_status spmv_autotune(maxe_handle* h, cudaStream_t st) {
   // the staged-tile kernel, when the handle has its tiles and it is clearly the
   // faster (on small matrices all take a launch, and a tie keeps the others)
   if (s == MAXE_OK && h->tiles) {
-    float ms = 0.f;
-    s = timed([&] { return spmv_tile_launch(h, x, y, nullptr, st); }, &ms);
-    h->tile_use = s == MAXE_OK && ms < 0.95f * best ? 1 : 0;
+    float sparse = 0.f, dense = 0.f;
+    s = timed([&] { return spmv_tile_launch(h, x, y, nullptr, st); }, &sparse);
+    h->tile_dense = 1;
+    if (s == MAXE_OK) s = timed([&] { return spmv_tile_launch(h, x, y, nullptr, st); }, &dense);
+    h->tile_dense = dense < sparse ? 1 : 0;
+    h->tile_use = s == MAXE_OK && std::min(sparse, dense) < 0.95f * best ? 1 : 0;
   }
   // SpMM path for wide right-hand sides, timed at k = 16 when the scratch is modest
   const int64_t k = 16;

@@ -22,8 +22,8 @@
 // G/s; 240 G/s reached while x stays in L2).  Permuted Laplacian, FP32, warp
 // kernel -> tiles: 4096 x 4096 646 -> 372 us (x of 67 MB no longer fits in L2
 // beside the stream), 2048 x 2048 97 -> 89 us; natural order, x in L1: 4096 x
-// 4096 215 -> 174 us, FP64 464 -> 271 us.  With longer rows (Poisson, 15 to 50
-// a row) the two are even and FP64 loses (150 -> 185 us at 20M entries), so the
+// 4096 215 -> 150 us, FP64 464 -> 268 us.  With longer rows (Poisson, 15 to 50
+// a row) the two are even, and the x-sliced form is faster where it applies, so the
 // autotuner times all and takes the tiles where they are 5% faster; a handle that
 // was not tuned keeps the warp kernel.
 #include <algorithm>
@@ -135,8 +135,18 @@ __device__ __forceinline__ void sts4(AT* p, const AT (&v)[4]) {
   }
 }
 
-template <typename VT, bool BIG>
-__global__ void __launch_bounds__(kTileThreads, 6) spmv_tile_kernel(const TileParams p) {
+// CTAs per SM a variant's registers are cut for.  Where x is gathered at random,
+// all gathers of a thread should be in flight and no more CTAs than that takes
+// (FP64 at six: 40 registers, two batches of gathers; permuted 3000 x 3000 Laplacian
+// 760 us, at four 331 us).  Where x is found in L1, more CTAs hide more (natural
+// 4096 x 4096, FP32: 172 us at six, 150 us at eight).  The autotuner times both.
+template <typename VT, bool DENSE>
+constexpr int tile_blocks() {
+  return sizeof(VT) == 8 ? (DENSE ? 6 : 4) : (DENSE ? 8 : 6);
+}
+
+template <typename VT, bool BIG, bool DENSE>
+__global__ void __launch_bounds__(kTileThreads, (tile_blocks<VT, DENSE>())) spmv_tile_kernel(const TileParams p) {
   using T = TileT<VT>;
   using AT = typename T::AT;
   __shared__ __align__(16) AT xs[kTileCap];
@@ -276,14 +286,11 @@ __global__ void tile_starts_kernel(const int32_t* __restrict__ first, const int3
   tile[b] = make_int2(r, rowptr[r]);
 }
 
-template <typename VT>
+template <typename VT, bool BIG>
 maxe_status tile_launch(const TileParams& p, const maxe_handle* h, cudaStream_t st) {
   const unsigned grid = static_cast<unsigned>(h->tiles);
-  if (beyond_l2(h, 1))
-    spmv_tile_kernel<VT, true><<<grid, kTileThreads, 0, st>>>(p);
-  else
-    spmv_tile_kernel<VT, false><<<grid, kTileThreads, 0, st>>>(p);
-  MAXE_CUDA_TRY(cudaGetLastError());
+  MAXE_CUDA_TRY(h->tile_dense ? launch_after(spmv_tile_kernel<VT, BIG, true>, grid, kTileThreads, 0, st, p)
+                              : launch_after(spmv_tile_kernel<VT, BIG, false>, grid, kTileThreads, 0, st, p));
   return MAXE_OK;
 }
 
@@ -314,10 +321,11 @@ maxe_status spmv_tile_build(maxe_handle* h, cudaStream_t st) {
 
 maxe_status spmv_tile_launch(const maxe_handle* h, const void* x, void* y, const int32_t* yperm, cudaStream_t st) {
   TileParams p{h->rowptr, h->col, h->val, h->tile, x, y, yperm, h->tile_shift};
+  const bool big = beyond_l2(h, 1);
   switch (h->dtype) {
-    case MAXE_F64: return tile_launch<double>(p, h, st);
-    case MAXE_F32: return tile_launch<float>(p, h, st);
-    case MAXE_BF16: return tile_launch<uint16_t>(p, h, st);
+    case MAXE_F64: return big ? tile_launch<double, true>(p, h, st) : tile_launch<double, false>(p, h, st);
+    case MAXE_F32: return big ? tile_launch<float, true>(p, h, st) : tile_launch<float, false>(p, h, st);
+    case MAXE_BF16: return big ? tile_launch<uint16_t, true>(p, h, st) : tile_launch<uint16_t, false>(p, h, st);
   }
   return MAXE_ERR_INVALID;
 }
