@@ -94,7 +94,8 @@ maxe_status gradient_permutation_run(const int32_t* hist, int32_t n, uint64_t se
   const int32_t half = (n + 1) / 2;
   ScratchSet scratch(al);
   int32_t* order = scratch.get<int32_t>(n);
-  void* tmp = scratch.get<unsigned char>(perm_order_scratch_bytes(half));
+  // for either half: the shorter one can ask for more (n = 2^23 + 1: 4096 buckets against 2048)
+  void* tmp = scratch.get<unsigned char>(std::max(perm_order_scratch_bytes(half), perm_order_scratch_bytes(n - half)));
   unsigned long long* best = scratch.get<unsigned long long>(1);
   if (!order || !tmp || !best) return MAXE_ERR_OOM;
   MAXE_CUDA_TRY(cudaMemsetAsync(best, 0, sizeof(unsigned long long), st));

@@ -93,6 +93,7 @@ inline bool beyond_l2(const maxe_handle* h, int64_t k) {
 }
 
 // perm.cu: out = first .. first + n - 1 in ascending (key(seed, tag, i), i) order.
+// The scratch is for that n alone: it does not always grow with n.
 size_t perm_order_scratch_bytes(int64_t n);
 maxe_status perm_order(uint64_t seed, int32_t tag, int32_t first, int32_t n, int32_t* out, void* scratch,
                        cudaStream_t st);
