@@ -67,7 +67,13 @@ typedef enum { MAXE_F64 = 0, MAXE_F32 = 1, MAXE_BF16 = 2 } maxe_dtype;
  * for the x-sliced form when the handle has one; also time the three SpMM
  * paths (column passes, columns across lanes, one row per lane group) at
  * k = 16 when their scratch (rows + cols) * 16 vectors fits in 8 GiB, and keep
- * the fastest (synchronises; a few products of device time). */
+ * the fastest (synchronises; a few products of device time).  SpMV by staged
+ * tiles (maxe_spmv_tiles) is timed too and kept where it is clearly faster; its
+ * table takes 8 bytes per tile of up to about 2000 entries.  With rperm and more
+ * than 30 MB of 16-byte rows (1.9 M rows) the handle also keeps the inverse of
+ * rperm and y' scratch, 20 bytes a row, for original-space products whose Y rows
+ * are at most 16 bytes and take more than 30 MB; without that memory such rows
+ * are scattered. */
 #define MAXE_AUTOTUNE 0x4u
 /* Flag of maxe_permute_csr: use the 16-entries-per-lane SpMV variant without
  * timing (tuning override; MAXE_AUTOTUNE takes precedence). */
@@ -284,7 +290,8 @@ MAXE_API maxe_status maxe_nnz_entropy_noalloc(const maxe_handle* h, int32_t gr, 
 /* a6 + a5.  y = A x (Section 2, CSR product) through the permuted matrix:
  * without MAXE_VEC_PERMUTED, x is gathered to x' = P_c^{-1} x in handle-owned
  * scratch, y' = A' x' is computed, and y[rperm[i']] = y'[i'] is written in the
- * product's epilogue, so y = A x.  With MAXE_VEC_PERMUTED, y = A' x directly.
+ * product's epilogue (on large autotuned handles by a second kernel, from y'
+ * scratch), so y = A x.  With MAXE_VEC_PERMUTED, y = A' x directly.
  * x: (device) cols elements, y: (device) rows elements; FP64 for MAXE_F64
  * handles, FP32 otherwise.  x and y must not overlap.  Calls on one handle
  * without MAXE_VEC_PERMUTED share its x' scratch (and the y' scratch of large

@@ -123,27 +123,31 @@ bool order_later(const maxe_handle* h, int64_t k) {
   return row <= kOrderRowBytes && row * h->rows > kOrderBytes;
 }
 
+// rinv and the y' scratch of such products, made with the handle and kept as long: a
+// call neither makes nor moves them, so a captured graph's addresses stay good.  Without
+// the memory rows are scattered.
+maxe_status order_later_build(maxe_handle* h, cudaStream_t st) {
+  if (!h->rperm || h->nnz == 0 || h->rows * kOrderRowBytes <= kOrderBytes) return MAXE_OK;
+  h->ybuf = h->al.get(static_cast<size_t>(h->rows) * kOrderRowBytes);
+  if (h->ybuf) h->rinv = static_cast<int32_t*>(h->al.get(static_cast<size_t>(h->rows) * sizeof(int32_t)));
+  if (!h->rinv) {
+    h->al.put(h->ybuf);
+    h->ybuf = nullptr;
+    return MAXE_OK;
+  }
+  MAXE_TRY(launch_invert(h->rperm, h->rows, h->rinv, st));
+  MAXE_CUDA_TRY(cudaStreamSynchronize(st));  // as all of an autotuned handle
+  return MAXE_OK;
+}
+
 // Y = P_r^{-1} A' X (rows through rperm).
 maxe_status product_original(const maxe_handle* h, int32_t k, const void* X, int64_t ldx, void* Y, int64_t ldy,
                              cudaStream_t st) {
-  if (!h->rinv || h->nnz == 0 || !order_later(h, k)) return spmm_launch(h, k, X, ldx, Y, ldy, h->rperm, st);
-  maxe_handle* hm = const_cast<maxe_handle*>(h);
-  const int32_t ld = k == 1 ? 1 : static_cast<int32_t>(round_up(k, 4));
-  if (hm->ybuf_k < ld) {  // without the scratch (none to be had, or not now): scattered
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    MAXE_CUDA_TRY(cudaStreamIsCapturing(st, &cap));
-    Allocator al = h->al;
-    al.stream = st;
-    void* p = cap == cudaStreamCaptureStatusNone
-                  ? al.get(static_cast<size_t>(h->rows) * static_cast<size_t>(ld) * vector_bytes(h->dtype))
-                  : nullptr;
-    if (!p) return spmm_launch(h, k, X, ldx, Y, ldy, h->rperm, st);
-    al.put(hm->ybuf);
-    hm->ybuf = p;
-    hm->ybuf_k = ld;
-  }
+  if (!h->rinv || !order_later(h, k)) return spmm_launch(h, k, X, ldx, Y, ldy, h->rperm, st);
+  const int eb = vector_bytes(h->dtype);
+  const int64_t ld = k == 1 ? 1 : kOrderRowBytes / eb;  // one element, or 16-byte rows
   MAXE_TRY(spmm_launch(h, k, X, ldx, h->ybuf, ld, nullptr, st));
-  return launch_gather(h->rinv, h->rows, vector_bytes(h->dtype), k, h->ybuf, ld, Y, ldy, st);
+  return launch_gather(h->rinv, h->rows, eb, k, h->ybuf, ld, Y, ldy, st);
 }
 
 }  // namespace
@@ -253,16 +257,13 @@ maxe_status maxe_permute_csr(const maxe_csr* A, const int32_t* rperm, const int3
     s = spmv_tile_build(h, st);
     if (s == MAXE_ERR_OOM) s = MAXE_OK;  // as above: the handle goes without it
   }
-  if (s == MAXE_OK && (flags & MAXE_AUTOTUNE) && h->rperm && h->rows * kOrderRowBytes > kOrderBytes) {
-    h->rinv = static_cast<int32_t*>(h->al.get(static_cast<size_t>(h->rows) * sizeof(int32_t)));
-    if (h->rinv) s = launch_invert(h->rperm, h->rows, h->rinv, st);  // without the memory: rows are scattered
-  }
   if (s == MAXE_OK) s = batch_plan_default(h, st);
   if (s == MAXE_OK && (flags & MAXE_ITEMS16)) h->spmv_items16 = 1;
   if (s == MAXE_OK && (flags & MAXE_SPMM_LANES)) h->spmm_lc = 1;
   if (s == MAXE_OK && (flags & MAXE_SPMM_ROWS)) h->spmm_rows = 1;
   if (s == MAXE_OK && (flags & MAXE_SPMM_ROWS_PF)) h->spmm_rows_pf = 1;
   if (s == MAXE_OK && (flags & MAXE_AUTOTUNE)) s = spmv_autotune(h, st);
+  if (s == MAXE_OK && (flags & MAXE_AUTOTUNE)) s = order_later_build(h, st);
   // the default batch plan follows the handle's SpMM path where it was tuned
   // or asked for, else takes the rows kernel
   if (s == MAXE_OK) h->blc = h->spmm_rows ? 2 : (h->spmm_lc ? 1 : ((flags & MAXE_AUTOTUNE) ? 0 : 2));

@@ -70,8 +70,7 @@ struct maxe_handle {
   void* xbuf = nullptr;  // cols * k_cap vector elements
   int32_t xbuf_k = 0;
   int32_t* rinv = nullptr;  // inverse of rperm, where Y rows may be put in order by a second pass
-  void* ybuf = nullptr;     // its y' scratch (original-space calls): rows * ybuf_k vector elements
-  int32_t ybuf_k = 0;
+  void* ybuf = nullptr;     // its y' scratch (original-space calls): 16 bytes a row
   maxe::Allocator al;
   int device = 0;
   int sms = 0;
