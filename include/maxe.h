@@ -335,7 +335,11 @@ MAXE_API maxe_status maxe_handle_coo(const maxe_handle* h, const int32_t** row);
 /* a7.  Y = A X for k right-hand sides (1 <= k <= 64).  X: (device) row-major
  * cols x k with leading dimension ldx >= k; Y: (device) row-major rows x k,
  * ldy >= k.  Element type and flags as for maxe_spmv.  Without
- * MAXE_VEC_PERMUTED, rows of X are gathered into handle-owned scratch.
+ * MAXE_VEC_PERMUTED, rows of X are gathered into handle-owned scratch, which
+ * holds four columns at first and grows, at least twofold, in the first call that
+ * needs more: make that call before one is captured in a CUDA graph.  Outgrown
+ * scratch stays until the handle is destroyed, so graphs captured earlier stay
+ * good.
  * Speed: with 16-byte aligned X and Y and ldx, ldy multiples of 4 (FP32) or 2
  * (FP64), rows are gathered 4 (2) columns per load, also when k is not a
  * multiple (the padding columns of X are read and ignored; Y's are untouched).

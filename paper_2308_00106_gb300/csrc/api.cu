@@ -1,6 +1,7 @@
 // api.cu -- the extern "C" entry points of libmaxe.so (declared in include/maxe.h).
 // Host-side argument checks, handle lifetime, and dispatch to the kernel
 // families; no arithmetic of the method runs here.
+#include <algorithm>
 #include <atomic>
 #include <mutex>
 #include <new>
@@ -80,6 +81,7 @@ void release(maxe_handle* h) {
   al.put(h->ybuf);
   al.put(h->rinv);
   al.put(h->xbuf);
+  for (int i = 0; i < h->xbuf_olds; ++i) al.put(h->xbuf_old[i]);
   xslice_release(h);
   al.put(h->tile);
   al.put(h->coo_carry);
@@ -95,15 +97,28 @@ void release(maxe_handle* h) {
   delete h;
 }
 
-// x' scratch for k right-hand sides (ld = round_up(k, 4)); grows on demand.
+constexpr int32_t kMaxColumns = 64;  // of maxe_spmm
+
+// Row stride (elements) of the x' scratch in a product with k columns: the call's own,
+// whatever the handle's products before it took.
+int64_t xbuf_stride(int32_t k) { return round_up(k, 4); }
+
+// x' scratch for k right-hand sides.  It grows on demand, twofold where the memory is
+// there, and the blocks that it outgrows stay with the handle (together less than the
+// last one then): a captured graph, or a call on another stream, may still use them.
 maxe_status ensure_xbuf(maxe_handle* h, int32_t k, cudaStream_t st) {
   if (h->xbuf && h->xbuf_k >= k) return MAXE_OK;
-  const int32_t kk = static_cast<int32_t>(round_up(k, 4));
   Allocator al = h->al;
   al.stream = st;
-  void* p = al.get(static_cast<size_t>(std::max(h->cols, 1)) * kk * vector_bytes(h->dtype));
+  auto get = [&](int32_t kk) {
+    return al.get(static_cast<size_t>(std::max(h->cols, 1)) * kk * vector_bytes(h->dtype));
+  };
+  const int32_t need = static_cast<int32_t>(xbuf_stride(k));
+  int32_t kk = std::max(need, std::min(2 * h->xbuf_k, kMaxColumns));
+  void* p = get(kk);
+  if (!p && kk > need) p = get(kk = need);
   if (!p) return MAXE_ERR_OOM;
-  al.put(h->xbuf);
+  if (h->xbuf) h->xbuf_old[h->xbuf_olds++] = h->xbuf;
   h->xbuf = p;
   h->xbuf_k = kk;
   return MAXE_OK;
@@ -370,7 +385,7 @@ maxe_status maxe_handle_coo(const maxe_handle* h, const int32_t** row) {
 
 maxe_status maxe_spmm(const maxe_handle* h, int32_t k, const void* X, int64_t ldx, void* Y, int64_t ldy,
                       uint32_t flags, void* stream) {
-  if (!h || k < 1 || k > 64 || ldx < k || ldy < k) return MAXE_ERR_INVALID;
+  if (!h || k < 1 || k > kMaxColumns || ldx < k || ldy < k) return MAXE_ERR_INVALID;
   if (flags & ~static_cast<uint32_t>(MAXE_VEC_PERMUTED)) return MAXE_ERR_INVALID;
   if ((h->cols > 0 && !X) || (h->rows > 0 && !Y)) return MAXE_ERR_INVALID;
   cudaStream_t st = as_stream(stream);
@@ -380,7 +395,7 @@ maxe_status maxe_spmm(const maxe_handle* h, int32_t k, const void* X, int64_t ld
   if (h->cperm) {
     maxe_handle* hm = const_cast<maxe_handle*>(h);
     MAXE_TRY(ensure_xbuf(hm, k, st));
-    lds = hm->xbuf_k;
+    lds = xbuf_stride(k);
     MAXE_TRY(launch_gather(h->cperm, h->cols, vector_bytes(h->dtype), k, X, ldx, hm->xbuf, lds, st));
     xs = hm->xbuf;
   }

@@ -67,8 +67,10 @@ struct maxe_handle {
   int xs_prefetch = 0;                     // cells large enough for the L2 prefetch cursor
   int32_t* coo_row = nullptr;              // COO row index of every entry (MAXE_COO), else NULL
   void* coo_carry = nullptr;               // COO per-chunk partial sums and flags
-  void* xbuf = nullptr;  // cols * k_cap vector elements
+  void* xbuf = nullptr;  // cols * xbuf_k vector elements
   int32_t xbuf_k = 0;
+  void* xbuf_old[16];    // the blocks that it outgrew (at least 4 of at most 64 columns a time)
+  int xbuf_olds = 0;
   int32_t* rinv = nullptr;  // inverse of rperm, where Y rows may be put in order by a second pass
   void* ybuf = nullptr;     // its y' scratch (original-space calls): 16 bytes a row
   maxe::Allocator al;
