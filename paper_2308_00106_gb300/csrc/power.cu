@@ -175,7 +175,8 @@ template <typename T>
 maxe_status run(const maxe_handle* h, const T* v0, int32_t steps, T* v, double* lambda_host, double* hist_host,
                 cudaStream_t st) {
   const int64_t n = h->rows;
-  ScratchSet scratch(h->al);
+  const Allocator al = h->al.on(st);
+  ScratchSet scratch(al);
   T* w = scratch.get<T>(static_cast<size_t>(n));
   T* xp = h->cperm ? scratch.get<T>(static_cast<size_t>(n)) : nullptr;
   double* part = scratch.get<double>(2 * kDotBlocks + 1 + (hist_host ? std::max(steps, 1) : 0));
