@@ -108,7 +108,7 @@ int64_t xbuf_stride(int32_t k) { return round_up(k, 4); }
 // last one then): a captured graph, or a call on another stream, may still use them.
 maxe_status ensure_xbuf(maxe_handle* h, int32_t k, cudaStream_t st) {
   if (h->xbuf && h->xbuf_k >= k) return MAXE_OK;
-  const Allocator al = h->al.on(st);
+  const Allocator al = allocator_on(h, st);
   auto get = [&](int32_t kk) {
     return al.get(static_cast<size_t>(std::max(h->cols, 1)) * kk * vector_bytes(h->dtype));
   };

@@ -280,7 +280,7 @@ int pick_vw(const maxe_batch_item& a, int eb) {
 maxe_status batch_plan(maxe_handle* h, int64_t H, int it16, cudaStream_t st, int lc, int bps) {
   H = std::max<int64_t>(256, H);
   const int64_t nW = std::max<int64_t>(1, ceil_div(h->nnz, H));
-  const Allocator al = h->al.on(st);
+  const Allocator al = allocator_on(h, st);
   int32_t* w = static_cast<int32_t*>(al.get(static_cast<size_t>(nW + 1) * sizeof(int32_t)));
   if (!w) return MAXE_ERR_OOM;
   maxe_status s = bucket_lower_bounds(h->rowptr, h->rows, H, 0, nW, w, st);
@@ -491,7 +491,7 @@ maxe_status maxe_batch_tune(maxe_handle* h, int32_t k, void* stream) {
   const int eb = vector_bytes(h->dtype);
   // rows padded to whole vectors, as callers are advised to lay X and Y out
   const int32_t kp = k == 1 ? 1 : static_cast<int32_t>(round_up(k, eb == 4 ? 4 : 2));
-  const Allocator al = h->al.on(st);
+  const Allocator al = allocator_on(h, st);
   ScratchSet scratch(al);
   void* X = scratch.get<unsigned char>(static_cast<size_t>(h->cols) * kp * eb);
   void* Y = scratch.get<unsigned char>(static_cast<size_t>(h->rows) * kp * eb);

@@ -84,6 +84,14 @@ namespace maxe {
 inline int value_bytes(maxe_dtype d) { return d == MAXE_F64 ? 8 : (d == MAXE_F32 ? 4 : 2); }
 inline int vector_bytes(maxe_dtype d) { return d == MAXE_F64 ? 8 : 4; }
 
+// The handle's allocator for a call on `st`: a block is free on the stream that it was
+// asked for, and may be in use on another.
+inline Allocator allocator_on(const maxe_handle* h, cudaStream_t st) {
+  Allocator al = h->al;
+  al.stream = st;
+  return al;
+}
+
 // Whether the arrays of a product with k columns leave no room to find them in L2
 // again (129 MB, of which a quarter is left to others): such a product streams
 // its matrix past x.

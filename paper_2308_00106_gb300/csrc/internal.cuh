@@ -184,13 +184,6 @@ struct Allocator {
       custom = true;
     }
   }
-  // The same allocator for a call on `s`: a block is free on the stream that it was
-  // asked for, and may be in use on another.
-  Allocator on(cudaStream_t s) const {
-    Allocator al = *this;
-    al.stream = s;
-    return al;
-  }
   void* get(size_t bytes) const {
     if (bytes == 0) bytes = 256;
     if (custom) return a.alloc(bytes, a.ctx, stream);

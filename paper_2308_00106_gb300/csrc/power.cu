@@ -175,7 +175,7 @@ template <typename T>
 maxe_status run(const maxe_handle* h, const T* v0, int32_t steps, T* v, double* lambda_host, double* hist_host,
                 cudaStream_t st) {
   const int64_t n = h->rows;
-  const Allocator al = h->al.on(st);
+  const Allocator al = allocator_on(h, st);
   ScratchSet scratch(al);
   T* w = scratch.get<T>(static_cast<size_t>(n));
   T* xp = h->cperm ? scratch.get<T>(static_cast<size_t>(n)) : nullptr;
