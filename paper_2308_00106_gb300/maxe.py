@@ -2,9 +2,11 @@
 
 Argument marshalling only: every step of the hot path runs in the library's
 CUDA kernels.  Torch provides device memory (its caching allocator is handed
-to the library as a ``maxe_allocator``) and the current CUDA stream.  There is
-no CPU fallback: if the library is missing or no GPU is visible, these calls
-raise.
+to the library as a ``maxe_allocator``) and the current CUDA stream.  A call
+with ``stream=`` takes its scratch on that stream; a result that it makes
+itself is a tensor of the current stream, as any other (pass the output to
+avoid that).  There is no CPU fallback: if the library is missing or no GPU is
+visible, these calls raise.
 
 Function names follow the C entry points.  Permutations use perm[new] = old
 (Eq. 1 of arXiv 2308.00106):  A' = P_r A P_c,  x' = x[cperm],  y[rperm] = y'.
@@ -77,22 +79,20 @@ class _Csr(ctypes.Structure):
 
 _lock = threading.Lock()
 _lib = None
-_live: dict[int, torch.Tensor] = {}  # allocations handed to the library
 
 
 def _torch_alloc(nbytes, ctx, stream):
+    """A block of torch's caching allocator that is free on `stream`, the call's own stream: a block of the
+    current stream's pool may still be in use by work pending there."""
     try:
-        t = torch.empty(max(int(nbytes), 1), dtype=torch.uint8, device="cuda")
+        return torch.cuda.caching_allocator_alloc(max(int(nbytes), 1), stream=stream or 0)
     except Exception:  # out of memory -> NULL -> MAXE_ERR_OOM
         return None
-    p = t.data_ptr()
-    _live[p] = t
-    return p
 
 
 def _torch_free(ptr, ctx, stream):
     if ptr:
-        _live.pop(int(ptr), None)
+        torch.cuda.caching_allocator_delete(ptr)
 
 
 _ALLOC = _Allocator(_Allocator._fields_[0][1](_torch_alloc), _Allocator._fields_[1][1](_torch_free), None)
