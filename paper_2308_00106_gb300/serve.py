@@ -21,10 +21,13 @@ about two steps per stream, so admitting interleaves with launching); each
 batch step takes one unit of work (a product) from
 admitted requests that are not already on the GPU, oldest first, up to a byte
 budget of work per step, so requests join and leave between steps and a power
-iteration advances one product per step -- or, while no other request waits to
-join, as many as the step's budget holds, in rounds one behind the other on the
-step's stream (a host round trip per product cost more than the product:
-two 20-step iterations on 300k-row matrices took most of a 7.5 ms trace).
+iteration advances one product per step -- or, while no other request has arrived,
+as many as the step's budget holds, in rounds one behind the other on the
+step's stream without the loop's polling between them (which cost more than the product:
+two 20-step iterations on 300k-row matrices took most of a 7.5 ms trace).  The loop
+looks for arrivals before each round.  Rounds of matrices in the x-sliced form are
+only queued; a batched round still waits on the host until the one before it is done,
+because it rewrites that one's staged table.
 Requests of one product are done after the first round.  Two CUDA streams, each with its own
 batch object, keep two steps in flight, so a step's work overlaps the previous
 one on the device.  Every matrix has a fixed
@@ -295,6 +298,8 @@ class Server:
                 products = len(take)
                 left = [r for r in take if r.units_done < r.units] if rounds else []
                 while left and work < self.step_bytes and products + len(left) <= cap_items:
+                    if nxt < n and trace[nxt].arrival <= time.perf_counter() - t0:
+                        break  # it joins before the iterations go on
                     self._launch(si, left)
                     more = sum(self.unit_bytes(r) for r in left)
                     work += more
