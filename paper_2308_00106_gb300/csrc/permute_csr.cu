@@ -47,7 +47,38 @@ struct SortSmem {
   uint32_t start[kSortCap / 32];  // bit per entry: a row starts here
   int32_t before[kSortCap / 32];  // last row start before this word
   uint32_t ws[kSortThreads / 32];
+  uint32_t pairs[kSortThreads / 32];
 };
+
+// Comparisons within bins (the sum of their squared counts) up to which a bucket is
+// ranked by bins.  On 25 M entries (12,200 buckets) 1000 comparisons in each take
+// 4.1 us and the sort takes 1050 us.
+constexpr uint32_t kMaxPairs = 250000;
+
+// Sorts sz keys (a power of two) in ascending order; the whole block.  Not inlined: its
+// registers are not the bins'.
+__device__ __noinline__ void sort_bucket(uint64_t* keys, int sz) {
+  for (int kk = 2; kk <= sz; kk <<= 1) {
+    for (int j = kk >> 1; j > 0; j >>= 1) {
+      for (int t = threadIdx.x; t < (sz >> 1); t += kSortThreads) {
+        const int lo = 2 * t - (t & (j - 1)), hi = lo + j;
+        const bool up = (lo & kk) == 0;
+        const uint64_t a = keys[lo], b = keys[hi];
+        if ((a > b) == up) {
+          keys[lo] = b;
+          keys[hi] = a;
+        }
+      }
+      __syncthreads();
+    }
+  }
+}
+
+// Start of the row that holds entry pos of the bucket.
+__device__ __forceinline__ int32_t row_of(const SortSmem& sm, int pos) {
+  const uint32_t bits = sm.start[pos >> 5] & (0xffffffffu >> (31 - (pos & 31)));
+  return bits ? (pos & ~31) + 31 - __clz(bits) : sm.before[pos >> 5];
+}
 
 // One CTA per bucket g: rows [first[g], first[g+1]) minus a trailing long row.
 //
@@ -56,9 +87,12 @@ struct SortSmem {
 // when not, where a row mostly is in order already): each entry counts itself
 // into its bin, a scan of all bins places the bins, and an entry's rank in its
 // bin is the number of smaller (column, position) pairs in it, of which there
-// are few.  Any columns are ordered right; uneven ones only make the bins
-// fuller (n^2 / 512 comparisons per thread at the worst).  A bitonic sort of
-// 64-bit keys took 1874 us for 25.4 M entries (2^20 rows), this took 417 us with two
+// are few.  Columns that crowd into few bins (a band under a column permutation that
+// keeps it, or one far column in rows that are otherwise close) would ask for up
+// to n^2 comparisons, so a bucket with more than kMaxPairs of them is sorted instead
+// (100,000 rows of 250 neighbours under an identity permutation, the whole call: 2579 us
+// ranked, 1507 us sorted; under a random one 490 us).
+// A bitonic sort of 64-bit keys took 1874 us for 25.4 M entries (2^20 rows), this took 417 us with two
 // CTAs an SM and takes 406 us with three (40 registers, a few spilled), with ten
 // barriers a bucket that leave a CTA waiting.
 template <typename VT>
@@ -121,8 +155,7 @@ __global__ void __launch_bounds__(kSortThreads, 3) bucket_sort_kernel(
   for (int u = 0; u < kSortItems; ++u) {
     const int pos = u * kSortThreads + static_cast<int>(threadIdx.x);
     if (pos < count) {
-      const uint32_t bits = sm.start[pos >> 5] & (0xffffffffu >> (31 - (pos & 31)));
-      row[u] = bits ? (pos & ~31) + 31 - __clz(bits) : sm.before[pos >> 5];
+      row[u] = row_of(sm, pos);
       const int32_t src = sm.a[row[u]] + pos;
       nc[u] = __ldcs(col + src);
       v[u] = __ldcs(val + src);
@@ -152,15 +185,19 @@ __global__ void __launch_bounds__(kSortThreads, 3) bucket_sort_kernel(
   for (int u = 0; u < kSortItems; ++u)
     if (u * kSortThreads + static_cast<int>(threadIdx.x) < count) atomicAdd(&sm.a[bin[u]], 1);
   __syncthreads();
-  {  // exclusive sums of the bins
+  {  // exclusive sums of the bins, and the comparisons that they ask for
     int4* pa = reinterpret_cast<int4*>(sm.a) + threadIdx.x * (kSortItems / 4);
     int4 w[kSortItems / 4];
     int32_t run = 0;
+    uint32_t pairs = 0;  // the block's total is at most kSortCap squared
 #pragma unroll
     for (int u = 0; u < kSortItems / 4; ++u) {
       w[u] = pa[u];
       run += w[u].x + w[u].y + w[u].z + w[u].w;
+      pairs += w[u].x * w[u].x + w[u].y * w[u].y + w[u].z * w[u].z + w[u].w * w[u].w;
     }
+    pairs = __reduce_add_sync(0xffffffffu, pairs);
+    if (lane == 0) sm.pairs[warp] = pairs;
     int32_t inc = run;
 #pragma unroll
     for (int d = 1; d < 32; d <<= 1) {
@@ -183,25 +220,50 @@ __global__ void __launch_bounds__(kSortThreads, 3) bucket_sort_kernel(
     }
   }
   __syncthreads();
-#pragma unroll
-  for (int u = 0; u < kSortItems; ++u) {  // into bin order; a[bin] ends as the bin's end
-    const int pos = u * kSortThreads + static_cast<int>(threadIdx.x);
-    if (pos < count) {
-      const int32_t p = atomicAdd(&sm.a[bin[u]], 1);
-      sm.b[p] = nc[u];
-      sm.c[p] = pos;
-    }
-  }
-  __syncthreads();
   int32_t rank[kSortItems];
+  if (__reduce_add_sync(0xffffffffu, sm.pairs[lane % (kSortThreads / 32)]) / 2 <= kMaxPairs) {
 #pragma unroll
-  for (int u = 0; u < kSortItems; ++u) {
-    const int pos = u * kSortThreads + static_cast<int>(threadIdx.x);
-    if (pos < count) {
-      const int32_t s = bin[u] ? sm.a[bin[u] - 1] : 0, e = sm.a[bin[u]];
-      rank[u] = s;
-      if (e - s > 1)
-        for (int32_t q = s; q < e; ++q) rank[u] += sm.b[q] < nc[u] || (sm.b[q] == nc[u] && sm.c[q] < pos);
+    for (int u = 0; u < kSortItems; ++u) {  // into bin order; a[bin] ends as the bin's end
+      const int pos = u * kSortThreads + static_cast<int>(threadIdx.x);
+      if (pos < count) {
+        const int32_t p = atomicAdd(&sm.a[bin[u]], 1);
+        sm.b[p] = nc[u];
+        sm.c[p] = pos;
+      }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < kSortItems; ++u) {
+      const int pos = u * kSortThreads + static_cast<int>(threadIdx.x);
+      if (pos < count) {
+        const int32_t s = bin[u] ? sm.a[bin[u] - 1] : 0, e = sm.a[bin[u]];
+        rank[u] = s;
+        if (e - s > 1)
+          for (int32_t q = s; q < e; ++q) rank[u] += sm.b[q] < nc[u] || (sm.b[q] == nc[u] && sm.c[q] < pos);
+      }
+    }
+  } else {
+    // Columns that share bins: all entries by (row start | new column | position), 55 bits.
+    uint64_t* keys = reinterpret_cast<uint64_t*>(sm.b);  // b and c
+    int sz = 1;
+    while (sz < count) sz <<= 1;
+#pragma unroll
+    for (int u = 0; u < kSortItems; ++u) {
+      const int pos = u * kSortThreads + static_cast<int>(threadIdx.x);
+      if (pos < count)
+        keys[pos] = (static_cast<uint64_t>(row_of(sm, pos)) << 43) | (static_cast<uint64_t>(nc[u]) << 12) |
+                    static_cast<uint64_t>(pos);
+      else if (pos < sz)
+        keys[pos] = ~0ull;
+    }
+    __syncthreads();
+    sort_bucket(keys, sz);
+    for (int p = threadIdx.x; p < count; p += kSortThreads) sm.a[keys[p] & 0xFFFull] = p;
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < kSortItems; ++u) {
+      const int pos = u * kSortThreads + static_cast<int>(threadIdx.x);
+      if (pos < count) rank[u] = sm.a[pos];
     }
   }
   __syncthreads();
