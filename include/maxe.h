@@ -124,9 +124,10 @@ typedef enum { MAXE_F64 = 0, MAXE_F32 = 1, MAXE_BF16 = 2 } maxe_dtype;
  * fastest). */
 #define MAXE_SPMM_ROWS 0x400u
 /* Flag of maxe_permute_csr: with MAXE_SPMM_ROWS, each lane group also
- * prefetches into L2 the X rows of its next row while it sums the current one
- * (tuning override; MAXE_AUTOTUNE times the rows kernel with and without it).
- * Results do not depend on it. */
+ * prefetches into L2 the X rows of its next row while it sums the current one,
+ * where a row takes more than one lane (tuning override, for every k;
+ * MAXE_AUTOTUNE times the rows kernel with and without it at k = 16 instead, and
+ * its pick acts from k = 16 on).  Results do not depend on it. */
 #define MAXE_SPMM_ROWS_PF 0x800u
 
 /* Device memory allocator used for everything a handle owns and for scratch.
@@ -237,9 +238,9 @@ MAXE_API maxe_status maxe_handle_csr(const maxe_handle* h, maxe_csr* view_out, c
  * group), plus in bits 15-17 the x-sliced form's L2 prefetch distance along
  * its entry stream in units of 512 entries (0: none; picked by MAXE_AUTOTUNE),
  * plus 0x40000 when the one-row-per-lane-group SpMM prefetches each lane
- * group's next X rows into L2 (picked by MAXE_AUTOTUNE: it pays where
- * neighbouring rows share X rows, as in a stencil, and costs on permuted
- * matrices), plus 0x80000 when maxe_spmv stages the gathered x of a tile of
+ * group's next X rows into L2 (MAXE_SPMM_ROWS_PF, or picked by MAXE_AUTOTUNE for
+ * k >= 16: it pays where neighbouring rows share X rows, as in a stencil, and
+ * mostly costs on permuted matrices), plus 0x80000 when maxe_spmv stages the gathered x of a tile of
  * rows in shared memory instead (picked by MAXE_AUTOTUNE; see maxe_spmv_tiles).  items: (host). */
 MAXE_API maxe_status maxe_handle_tuning(const maxe_handle* h, int32_t* items);
 

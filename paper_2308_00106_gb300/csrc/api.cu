@@ -275,7 +275,7 @@ maxe_status maxe_permute_csr(const maxe_csr* A, const int32_t* rperm, const int3
   if (s == MAXE_OK && (flags & MAXE_ITEMS16)) h->spmv_items16 = 1;
   if (s == MAXE_OK && (flags & MAXE_SPMM_LANES)) h->spmm_lc = 1;
   if (s == MAXE_OK && (flags & MAXE_SPMM_ROWS)) h->spmm_rows = 1;
-  if (s == MAXE_OK && (flags & MAXE_SPMM_ROWS_PF)) h->spmm_rows_pf = 1;
+  if (s == MAXE_OK && (flags & MAXE_SPMM_ROWS_PF)) h->spmm_rows_pf = 2;
   if (s == MAXE_OK && (flags & MAXE_AUTOTUNE)) s = spmv_autotune(h, st);
   if (s == MAXE_OK && (flags & MAXE_AUTOTUNE)) s = order_later_build(h, st);
   // the default batch plan follows the handle's SpMM path where it was tuned

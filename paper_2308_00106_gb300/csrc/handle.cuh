@@ -31,7 +31,7 @@ struct maxe_handle {
   int spmv_items16 = 0;                    // chosen SpMV variant (autotuned or 0)
   int spmm_lc = 0;                         // SpMM with columns across lanes (autotuned or 0)
   int spmm_rows = 0;                       // SpMM with one row per lane group (autotuned or 0)
-  int spmm_rows_pf = 0;                    // that kernel prefetches each group's next X rows (autotuned)
+  int spmm_rows_pf = 0;                    // that kernel prefetches each group's next X rows: 1 autotuned, 2 asked for
   int equal_rows = 0;                      // SpMV partition: equal rows per warp (not equal nonzeros)
   int2* tile = nullptr;                    // staged-tile SpMV (MAXE_AUTOTUNE): [tiles + 1] first row, its first entry
   int64_t tiles = 0;

@@ -226,10 +226,10 @@ maxe_status spmm_rows_launch(const maxe_handle* h, int32_t k, const void* X, int
   p.op.ldx = ldx;
   p.op.ldy = ldy;
   p.op.k = k;
-  // From k = 16 on, where the autotuner timed it: narrower rows lose by it (natural
-  // 2048 x 2048 Laplacian, FP32, k = 8: 114 us with, 110 without; permuted 4096 x
-  // 4096, FP64, k = 4: 2750 and 1902 us).
-  p.op.pf = h->spmm_rows_pf && k >= 16;
+  // The autotuner's pick acts from k = 16 on, where it was timed: narrower rows lose by
+  // it (natural 2048 x 2048 Laplacian, FP32, k = 8: 114 us with, 110 without; permuted
+  // 4096 x 4096, FP64, k = 4: 2750 and 1932 us).  A caller's own flag acts on any k.
+  p.op.pf = h->spmm_rows_pf == 2 || (h->spmm_rows_pf == 1 && k >= 16);
   p.once = !h->spmm_rows_pf && beyond_l2(h, k);
   p.wrow = h->wrow[0];
   p.nW = h->nW[0];
