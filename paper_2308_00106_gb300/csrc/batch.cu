@@ -153,7 +153,7 @@ __global__ void __launch_bounds__(kThreads, 3) spmm_batch_rows_kernel(BatchParam
     const rows::RowsOperand op{it.rowptr, it.col, it.val, it.X, it.Y, it.yperm, it.ldx, it.ldy, it.k, 0};
     const int w = t - bp.task0[lo];
     const int32_t ra = it.wrow[w], rb = it.wrow[w + 1];
-    constexpr int VC = rows::RowsT<VT>::kLaneCols;
+    constexpr int VC = rows::RowsT<VT>::VC;
     const int G = rows::rows_lanes((it.k + VC - 1) / VC);
     switch (G) {
       case 1: rows::rows_range<VT, VC, (VC > 1), 1>(s, op, ra, rb, G, lane); break;

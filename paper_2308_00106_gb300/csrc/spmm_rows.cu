@@ -2,11 +2,11 @@
 // product, k right-hand sides): one row per group of G lanes, single-matrix
 // launch (the per-warp machinery is in spmm_rows.cuh).
 //
-// Each lane holds VC = 16 bytes of columns of X and Y (4 FP32 / 2 FP64), so a
-// group of G lanes covers G * VC columns (more columns: more passes over the
-// row).  A group walks its row's entries, gathers the 16-byte piece of X row
-// COL that is its lanes', accumulates in registers and writes its piece of Y
-// once.
+// Each lane holds a piece of VC columns of X and Y (FP32: 16 bytes; FP64: one
+// column, see RowsT), so a group of G lanes covers G * VC columns (more columns:
+// more passes over the row).  A group walks its row's entries, gathers the piece of
+// X row COL that is its lanes', accumulates in registers and writes its piece of
+// Y once.
 //
 // The row's column indices come from shared memory, so that the gathers of X
 // (the bytes that matter) are the only global loads a row waits for.  A warp
@@ -33,11 +33,12 @@
 // keeps this path only for matrices where it is faster.  Requires 16-byte
 // aligned column and value arrays and rows of X under 2 GiB.
 //
-// X or Y rows that are not whole 16-byte pieces (an odd k in contiguous
-// tensors) take a variant whose lanes load 16, 8 or 4 (FP64: 8) bytes, as X's
-// alignment allows, with up to 32 lanes to a row, and store Y column by column: an X row is still read by one load of the group.  Poisson rows of
-// 20, 100,003 rows, FP32, k = 7 contiguous: 58 us in seven column passes, 21 us
-// here (k = 31: 236 -> 42 us; FP64, k = 7: 131 -> 69 us).
+// FP32 rows of X or Y that are not whole 16-byte pieces (an odd k in contiguous
+// tensors) take a variant whose lanes load 16, 8 or 4 bytes, as X's alignment
+// allows, with up to 32 lanes to a row, and store Y column by column: an X row is
+// still read by one load of the group.  Poisson rows of 20, 100,003 rows, FP32, k = 7
+// contiguous: 59 us in seven column passes, 19 us here (k = 31: 237 -> 36 us; FP64,
+// k = 7: 132 -> 58 us).
 #include "launch.cuh"
 #include "spmm_rows.cuh"
 
@@ -178,7 +179,7 @@ maxe_status launch_rows(RowsParams p, int sms, cudaStream_t st) {
   auto whole = [](const void* q, int64_t ld, int vc) {
     return ld % vc == 0 && reinterpret_cast<uintptr_t>(q) % (vc * sizeof(AT)) == 0;
   };
-  if constexpr (RowsT<VT>::kLaneCols == 1) {  // FP64: see there
+  if constexpr (VC == 1) {  // FP64: see RowsT
     switch (rows_lanes(p.op.k)) {
       case 1: return launch_rows_g<VT, 1, 1, false>(p, sms, st);
       case 2: return launch_rows_g<VT, 2, 1, false>(p, sms, st);

@@ -33,27 +33,24 @@ struct RowsT;
 template <>
 struct RowsT<float> {
   using AT = float;
-  static constexpr int VC = 4;         // columns of a 16-byte piece
-  static constexpr int kLaneCols = 4;  // columns a lane takes of aligned rows
+  static constexpr int VC = 4;  // columns a lane takes of 16-byte aligned rows
   static __device__ __forceinline__ float acc(float v) { return v; }
 };
 template <>
 struct RowsT<uint16_t> {
   using AT = float;
   static constexpr int VC = 4;
-  static constexpr int kLaneCols = 4;
   static __device__ __forceinline__ float acc(uint16_t v) { return __uint_as_float(static_cast<uint32_t>(v) << 16); }
 };
 template <>
 struct RowsT<double> {
   using AT = double;
-  static constexpr int VC = 2;
   // One column a lane whatever the alignment: twice the lanes a row, so half the
   // rows a warp, which costs fewer bank conflicts of the staged entries and less
   // waiting for the longest row than 16-byte loads save.  300,000 rows of 40, k = 4:
   // 352 -> 184 us, k = 16: 604 -> 436 us; permuted 2048 x 2048 Laplacian 534 -> 397
   // and 1300 -> 1250 us.
-  static constexpr int kLaneCols = 1;
+  static constexpr int VC = 1;
   static __device__ __forceinline__ double acc(double v) { return v; }
 };
 
@@ -73,10 +70,6 @@ struct RowsPiece<float, 1> {
   using V = float;
 };
 template <>
-struct RowsPiece<double, 2> {
-  using V = double2;
-};
-template <>
 struct RowsPiece<double, 1> {
   using V = double;
 };
@@ -93,19 +86,11 @@ __device__ __forceinline__ void fma_vec(float2& acc, float a, const float2& x) {
 }
 __device__ __forceinline__ void fma_vec(float& acc, float a, float x) { acc = fmaf(a, x, acc); }
 __device__ __forceinline__ void fma_vec(double& acc, double a, double x) { acc = fma(a, x, acc); }
-__device__ __forceinline__ void fma_vec(double2& acc, double a, const double2& x) {
-  acc.x = fma(a, x.x, acc.x);
-  acc.y = fma(a, x.y, acc.y);
-}
 __device__ __forceinline__ void add_vec(float4& a, const float4& b) {
   a.x += b.x;
   a.y += b.y;
   a.z += b.z;
   a.w += b.w;
-}
-__device__ __forceinline__ void add_vec(double2& a, const double2& b) {
-  a.x += b.x;
-  a.y += b.y;
 }
 __device__ __forceinline__ void add_vec(float2& a, const float2& b) {
   a.x += b.x;
@@ -124,13 +109,6 @@ __device__ __forceinline__ void store_piece(float4* y, const float4& v, int left
   if (left > 1) f[1] = v.y;
   if (left > 2) f[2] = v.z;
 }
-__device__ __forceinline__ void store_piece(double2* y, const double2& v, int left) {
-  if (left >= 2) {
-    *y = v;
-    return;
-  }
-  reinterpret_cast<double*>(y)[0] = v.x;
-}
 // Y rows that are not 16-byte aligned: column by column
 template <typename AT, typename V>
 __device__ __forceinline__ void store_columns(AT* y, const V& v, int left) {
@@ -143,7 +121,6 @@ __device__ __forceinline__ void zero(float2& v) { v = make_float2(0.f, 0.f); }
 __device__ __forceinline__ void zero(float& v) { v = 0.f; }
 __device__ __forceinline__ void zero(double& v) { v = 0.0; }
 __device__ __forceinline__ void zero(float4& v) { v = make_float4(0.f, 0.f, 0.f, 0.f); }
-__device__ __forceinline__ void zero(double2& v) { v = make_double2(0.0, 0.0); }
 
 // ONCE: the bytes are the first to leave L2.
 template <bool ONCE>
