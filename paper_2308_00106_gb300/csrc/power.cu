@@ -163,9 +163,11 @@ unsigned scale_blocks(int64_t n) {
   return static_cast<unsigned>(std::max<int64_t>(1, ceil_div(n, kDotThreads * kScaleItems)));
 }
 
-// The products of an iteration keep one order of sums whatever the tile rule
-// does: a quotient of a matrix without a dominant eigenvalue moves by 1e-6 with
-// the order of its FP32 products, far more than with anything else here.
+// The products of an iteration are never staged tiles, so that its history does not
+// move with what the autotuner picked: the quotient of a matrix without a dominant
+// eigenvalue moves by 1e-6 with the order of its FP32 sums, as with any change of
+// rounding.  A large permuted stencil pays for it (4096 x 4096, FP32: a product takes
+// 660 us here and 377 us by tiles).
 constexpr int kProduct = -2;
 
 // hist_host (nullable): the Rayleigh quotient v^T A v of the iterate after

@@ -262,11 +262,14 @@ maxe_status spmv_autotune(maxe_handle* h, cudaStream_t st) {
     best = std::min(best, best_xs);
   }
   // The staged-tile kernel, when the handle has its tiles and it is clearly the
-  // faster: by 5% over the CSR kernel; by 15% over the x-sliced form, and not on
-  // small matrices, where both take a launch and the timing is chance -- the served
-  // iterations of such a handle keep the order of the x-sliced sums.  (Poisson
-  // rows, the x-sliced form's own: tiles 4% slower at 2M entries, 60% at 6M.  A
-  // natural 1000 x 1000 Laplacian: 30% faster.)
+  // faster: by 5% over the CSR kernel; by 15% over the x-sliced form (Poisson rows,
+  // that form's own: tiles 4% slower at 2M entries, 60% at 6M; a natural 1000 x 1000
+  // Laplacian: 30% faster).  Below 2^20 nonzeros the x-sliced form stays without a
+  // comparison: launched one by one both take a launch here, so the choice, and with it
+  // the bits of the result, would fall by chance.  Replayed from a graph tiles would
+  // gain on stencils (natural 300 x 300, FP32: 4.5 and 2.9 us; 450 x 450: 4.5 and 3.3),
+  // less on power-law rows (40,000 permuted: 9.2 and 7.3 us), and lose on some (FP64,
+  // natural: 11.0 and 13.2 us).
   if (s == MAXE_OK && h->tiles) {
     float sparse = 0.f, dense = 0.f;
     s = timed([&] { return spmv_tile_launch(h, x, y, nullptr, st); }, &sparse);

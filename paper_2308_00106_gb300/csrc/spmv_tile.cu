@@ -1,5 +1,7 @@
 // spmv_tile.cu -- SpMV for matrices with short rows: y' = A' x' (Section 2's
-// CSR product) with the gathered x of a tile staged in shared memory.
+// CSR product) with the gathered x of a tile staged in shared memory.  Staging a
+// block of whole rows entry by entry and summing the rows from there is the
+// CSR-stream idea (Greathouse and Daga, SC 2014).
 //
 // The warp kernel of spmv.cu sums rows by a segmented scan over its entries
 // and reads every row end back from it: about a quarter of a millisecond of
