@@ -244,7 +244,6 @@ size_t radix_scratch_bytes(int64_t n);
 // in keys/vals (the *_alt buffers are ping-pong space).
 maxe_status radix_sort_pairs(uint64_t* keys, int32_t* vals, uint64_t* keys_alt, int32_t* vals_alt,
                              int64_t n, int bits, void* scratch, cudaStream_t st);
-maxe_status launch_keys(uint64_t seed, int32_t n, int32_t tag, uint64_t* keys, int32_t* idx, cudaStream_t st);
 maxe_status launch_invert(const int32_t* perm, int32_t n, int32_t* inv, cudaStream_t st);
 maxe_status launch_gather(const int32_t* perm, int64_t n, int elem_bytes, int64_t row_elems, const void* in,
                           int64_t ld_in, void* out, int64_t ld_out, cudaStream_t st);
