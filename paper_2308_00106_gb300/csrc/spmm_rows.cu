@@ -89,15 +89,17 @@ constexpr int rows_blocks() {
   return sizeof(AT) == 8 ? 3 : 4;
 }
 
-// The matrix leaves L2 first (ONCE), so that X stays: where columns were permuted, so
-// that X rows are gathered at random, and the product does not fit in L2.  Permuted 2048
-// x 2048 Laplacian, without and with it: FP32 k = 4 151 and 136 us, k = 8 262 and 251,
-// k = 16 392 and 386; BF16 k = 4 122 and 113, k = 16 406 and 402; FP64 k = 2 217 and 200,
-// k = 4 394 and 387, k = 8 690 and 690, k = 12 1257 and 1263: hence X rows of up to 64
-// bytes.  A stencil's X rows are in L2 anyway, and its product is up to 2% slower so
-// (FP32, k = 4: 71.2 and 73.0 us).  Rows of FP32 vectors that are not 16-byte pieces go
-// without: they were not timed with it.
-constexpr int64_t kOnceRowBytes = 64;
+// The matrix leaves L2 first (ONCE), so that X stays, where the product does not fit in
+// L2.  Columns permuted, so that X rows are gathered at random: 2048 x 2048 Laplacian,
+// without and with it, FP32 k = 4 151 and 136 us, k = 8 262 and 251, k = 16 392 and 386;
+// BF16 k = 4 122 and 113, k = 16 406 and 402; FP64 k = 2 217 and 200, k = 4 394 and 387,
+// k = 8 690 and 690, k = 12 1257 and 1263: hence X rows of up to 64 bytes.  In natural
+// order, FP32: k = 4 71.2 and 73.0, k = 8 107 and 108, k = 12 177 and 172, k = 16 189.5
+// and 186.8, k = 32 376 and 372: hence rows of more than 32 bytes, unless the prefetch
+// was kept, which gains as much.  FP32 rows that are not 16-byte
+// pieces go without: they were not timed with it.
+constexpr int64_t kOnceRandomMax = 64;
+constexpr int64_t kOnceOrderedMin = 32;
 
 // GC: lanes per row (0: p.G, a power of two; a constant is worth 10% on rows of
 // 40); VC, YVEC: see rows_chunk; ONCE: above.
@@ -237,7 +239,8 @@ maxe_status spmm_rows_launch(const maxe_handle* h, int32_t k, const void* X, int
   // it (natural 2048 x 2048 Laplacian, FP32, k = 8: 114 us with, 110 without; permuted
   // 4096 x 4096, FP64, k = 4: 2750 and 1932 us).  A caller's own flag acts on any k.
   p.op.pf = h->spmm_rows_pf == 2 || (h->spmm_rows_pf == 1 && k >= 16);
-  p.once = h->cperm && k * vector_bytes(h->dtype) <= kOnceRowBytes && beyond_l2(h, k);
+  const int64_t xrow = k * vector_bytes(h->dtype);
+  p.once = (h->cperm ? xrow <= kOnceRandomMax : xrow > kOnceOrderedMin && !h->spmm_rows_pf) && beyond_l2(h, k);
   p.wrow = h->wrow[0];
   p.nW = h->nW[0];
   // parts of about kPartE entries: a warp's range cut into Q parts of equal row counts
